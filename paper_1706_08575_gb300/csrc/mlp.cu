@@ -13,10 +13,9 @@
 // be closer), so the neighbour sets are exact.
 // MLP: BF16 tensor-core mma.sync m16n8k16 with FP32 accumulation; one warp owns 16 rows, and the
 // FP32 accumulator fragment of one layer is repacked in registers as the A fragment of the next.
-// Training: forward (activations kept), a row-wise backward that produces dz3, dz2, dz1 with the
-// same MMAs against the untransposed weights, a weight-gradient kernel that reduces act^T dz over
-// the batch with MMAs (activations staged transposed in shared memory), and Adam on an FP32
-// master copy.
+// Training: one kernel per step runs forward, backward and the weight gradients of 64 rows at a time
+// without leaving shared memory, and writes per-CTA partial gradients; a second one sums them in a
+// fixed order and applies Adam to an FP32 master copy.
 
 #include <cmath>
 #include <cstring>
@@ -257,22 +256,22 @@ __device__ __forceinline__ float gelu(float z) {
     return 0.5f * z * (1.0f + tanhf(c * (z + 0.044715f * z * z * z)));
 }
 
-__device__ __forceinline__ float gelu_grad(float z) {
+// gelu(z) and its derivative, sharing the tanh
+__device__ __forceinline__ float gelu_with_grad(float z, float* grad) {
     const float c = 0.7978845608028654f;
     const float t = tanhf(c * (z + 0.044715f * z * z * z));
-    return 0.5f * (1.0f + t) + 0.5f * z * (1.0f - t * t) * c * (1.0f + 3.0f * 0.044715f * z * z);
+    *grad = 0.5f * (1.0f + t) + 0.5f * z * (1.0f - t * t) * c * (1.0f + 3.0f * 0.044715f * z * z);
+    return 0.5f * z * (1.0f + t);
 }
 
-// BF16 weights in shared memory: forward layout Wt[out][in] (B fragment pairs along in), backward
-// layout Wn[in][out] (pairs along out), biases and w4 in FP32.
+// BF16 weights in shared memory, Wt[out][in] (B fragment pairs along in); biases and w4 in FP32.
 struct MlpSmem {
     __nv_bfloat16 w1t[kHid * kLd1];
     __nv_bfloat16 w2t[kHid * kLdH], w3t[kHid * kLdH];
-    __nv_bfloat16 w2n[kHid * kLdH], w3n[kHid * kLdH];
     float b1[kHid], b2[kHid], b3[kHid], w4[kHid], b4;
 };
 
-__device__ void load_smem(MlpSmem& s, const float* __restrict__ P, bool backward) {
+__device__ void load_smem(MlpSmem& s, const float* __restrict__ P) {
     for (int i = threadIdx.x; i < kHid * kLd1; i += blockDim.x) {
         const int o = i / kLd1, k = i % kLd1;
         s.w1t[i] = __float2bfloat16_rn(k < kIn ? P[oW1 + k * kHid + o] : 0.f);
@@ -282,10 +281,6 @@ __device__ void load_smem(MlpSmem& s, const float* __restrict__ P, bool backward
         const bool ok = c < kHid;
         s.w2t[i] = __float2bfloat16_rn(ok ? P[oW2 + c * kHid + r] : 0.f);
         s.w3t[i] = __float2bfloat16_rn(ok ? P[oW3 + c * kHid + r] : 0.f);
-        if (backward) {
-            s.w2n[i] = __float2bfloat16_rn(ok ? P[oW2 + r * kHid + c] : 0.f);
-            s.w3n[i] = __float2bfloat16_rn(ok ? P[oW3 + r * kHid + c] : 0.f);
-        }
     }
     for (int i = threadIdx.x; i < kHid; i += blockDim.x) {
         s.b1[i] = P[ob1 + i];
@@ -313,30 +308,13 @@ __device__ __forceinline__ void gemm_rows(float (*acc)[4], const uint32_t (*a)[4
         }
 }
 
-// bias (+) then GELU on the accumulators; z saved (training); A fragments of the next layer
-__device__ __forceinline__ void act_layer(float (*acc)[4], uint32_t (*anext)[4], float* zsave,
-                                          __nv_bfloat16* hsave, int64_t r0, int64_t M, int g,
-                                          int t) {
+// GELU on the accumulators; A fragments of the next layer
+__device__ __forceinline__ void act_layer(float (*acc)[4], uint32_t (*anext)[4]) {
     float h[8][4];
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
         for (int q = 0; q < 4; ++q) h[nt][q] = bf16r(gelu(acc[nt][q]));
-    if (zsave) {
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                const int64_t row = r0 + g + 8 * hh;
-                if (row < M) {
-                    const int col = 8 * nt + 2 * t;
-                    zsave[row * kHid + col] = acc[nt][2 * hh];
-                    zsave[row * kHid + col + 1] = acc[nt][2 * hh + 1];
-                    hsave[row * kHid + col] = __float2bfloat16_rn(h[nt][2 * hh]);
-                    hsave[row * kHid + col + 1] = __float2bfloat16_rn(h[nt][2 * hh + 1]);
-                }
-            }
-    }
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
         anext[kk][0] = pack_bf16(h[2 * kk][0], h[2 * kk][1]);
@@ -344,8 +322,6 @@ __device__ __forceinline__ void act_layer(float (*acc)[4], uint32_t (*anext)[4],
         anext[kk][2] = pack_bf16(h[2 * kk + 1][0], h[2 * kk + 1][1]);
         anext[kk][3] = pack_bf16(h[2 * kk + 1][2], h[2 * kk + 1][3]);
     }
-    if (!zsave) return;
-    (void)hsave;
 }
 
 __device__ __forceinline__ void init_bias(float (*acc)[4], const float* b, int t) {
@@ -356,18 +332,13 @@ __device__ __forceinline__ void init_bias(float (*acc)[4], const float* b, int t
     }
 }
 
-// Forward: rows idx[r] (or r) of X; y = log alpha. With TRAIN the pre-activations z1..z3 (FP32)
-// and activations h1..h3 (BF16) of batch row r are stored at row r.
-template <bool TRAIN>
+// alpha = exp(y) of every feature row.
 __global__ void __launch_bounds__(128)
-    k_mlp_forward(const __nv_bfloat16* __restrict__ X, const int* __restrict__ idx, int64_t M,
-                  const float* __restrict__ P, float* __restrict__ y, double* __restrict__ alpha,
-                  float* __restrict__ z1, float* __restrict__ z2, float* __restrict__ z3,
-                  __nv_bfloat16* __restrict__ h1, __nv_bfloat16* __restrict__ h2,
-                  __nv_bfloat16* __restrict__ h3) {
+    k_mlp_forward(const __nv_bfloat16* __restrict__ X, int64_t M, const float* __restrict__ P,
+                  double* __restrict__ alpha) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     MlpSmem& s = *reinterpret_cast<MlpSmem*>(smem_raw);
-    load_smem(s, P, false);
+    load_smem(s, P);
     __syncthreads();
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -379,8 +350,7 @@ __global__ void __launch_bounds__(128)
         for (int hh = 0; hh < 2; ++hh) {
             const int64_t row = r0 + g + 8 * hh;
             const bool ok = row < M;
-            const int64_t src = ok ? (idx ? (int64_t)idx[row] : row) : 0;
-            const __nv_bfloat16* xr = X + src * kInPad;
+            const __nv_bfloat16* xr = X + (ok ? row : 0) * kInPad;
 #pragma unroll
             for (int kk = 0; kk < 3; ++kk) {
                 a1[kk][hh] = ok ? ld32(xr + 16 * kk + 2 * t) : 0u;
@@ -391,13 +361,13 @@ __global__ void __launch_bounds__(128)
         uint32_t an[4][4];
         init_bias(acc, s.b1, t);
         gemm_rows<3>(acc, a1, s.w1t, kLd1, g, t);
-        act_layer(acc, an, TRAIN ? z1 : nullptr, h1, r0, M, g, t);
+        act_layer(acc, an);
         init_bias(acc, s.b2, t);
         gemm_rows<4>(acc, an, s.w2t, kLdH, g, t);
-        act_layer(acc, an, TRAIN ? z2 : nullptr, h2, r0, M, g, t);
+        act_layer(acc, an);
         init_bias(acc, s.b3, t);
         gemm_rows<4>(acc, an, s.w3t, kLdH, g, t);
-        act_layer(acc, an, TRAIN ? z3 : nullptr, h3, r0, M, g, t);
+        act_layer(acc, an);
         // output layer in FP32 on the BF16-rounded h3 (the A fragments hold exactly those values)
         float part[2] = {0.f, 0.f};
 #pragma unroll
@@ -420,209 +390,299 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
                 const int64_t row = r0 + g + 8 * hh;
-                if (row < M) {
-                    const float yy = part[hh] + s.b4;
-                    if (y) y[row] = yy;
-                    if (alpha) alpha[row] = exp((double)yy);
-                }
+                if (row < M) alpha[row] = exp((double)(part[hh] + s.b4));
             }
     }
 }
 
-// Row-wise backward of the mean squared error: dy -> dz3 -> dz2 -> dz1 (BF16, row-major), loss.
-__global__ void __launch_bounds__(128)
-    k_mlp_backward(const double* __restrict__ target, const int* __restrict__ idx, int64_t B,
-                   const float* __restrict__ P, const float* __restrict__ y,
-                   const float* __restrict__ z1, const float* __restrict__ z2,
-                   const float* __restrict__ z3, float* __restrict__ dy,
-                   __nv_bfloat16* __restrict__ dz1, __nv_bfloat16* __restrict__ dz2,
-                   __nv_bfloat16* __restrict__ dz3, float* __restrict__ loss) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    MlpSmem& s = *reinterpret_cast<MlpSmem*>(smem_raw);
-    load_smem(s, P, true);
-    __syncthreads();
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    float lsum = 0.f;
-    for (int64_t tile = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-         tile * 16 < B; tile += nwarps) {
-        const int64_t r0 = tile * 16;
-        float d[2];
+// ---------------------------------------------------------------------------------------------
+// Training: forward, backward and weight gradients of 64 rows by one CTA of 8 warps.
+//
+// Warp (rg, hf) = (warp & 3, warp >> 2) owns rows 16 rg .. 16 rg + 15 and half hf of the 64 columns of
+// every layer, so that a layer costs a thread 16 activations. The BF16 rows of X, h1..h3 and
+// dz3..dz1 stay in shared memory, where ldmatrix reads them as A operands of the next product
+// (straight) and as both operands of act^T dz (transposed); one copy Wt[out][in] of each weight
+// serves the forward product (straight) and dh = dz W^T (transposed). gelu'(z) is kept in registers
+// from the forward pass. The weight gradients accumulate in the MMA fragments over all tiles of the
+// CTA. Bound: the chain of 13 dependent phases of one tile, not bytes (about 1 MB of X per step at
+// B = 8192) or tensor rate; hence small tiles (128 CTAs at B = 8192) and everything in one launch.
+// Measured at B = 8192, us per step: separate forward, backward, per-layer weight-gradient kernels
+// of 8 CTAs each and serial reductions 571; this kernel and k_mlp_update 18.2 (B = 200,000: 1231
+// and 144).
+constexpr int kTrainRows = 64, kTrainThreads = 256;
+constexpr int kPartStride = (kParams + 1 + 31) / 32 * 32;   // packed gradients, then the loss
+
+struct TrainSmem {
+    __nv_bfloat16 x[kTrainRows * kLd1];
+    __nv_bfloat16 h[3][kTrainRows * kLdH];     // h1..h3
+    __nv_bfloat16 dz[3][kTrainRows * kLdH];    // dz1..dz3
+    __nv_bfloat16 w1t[kHid * kLd1];
+    __nv_bfloat16 w2t[kHid * kLdH], w3t[kHid * kLdH];
+    float bias[3][kHid], w4[kHid];
+    float ypart[2][kTrainRows], target[kTrainRows], dy[kTrainRows];
+    float small[4][5][kHid];
+    float b4;
+};
+
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const __nv_bfloat16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const __nv_bfloat16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+}
+
+// acc[4][4] += A(rows 16 rg .., KSTEPS k-steps, row stride LDA) * W(columns 32 hf ..), W from
+// wt[out][in] (forward, LDW) or, TRANS, from wt[out][in] as W^T (backward: k = out, n = in).
+template <int KSTEPS, int LDA, int LDW, bool TRANS>
+__device__ __forceinline__ void train_gemm(float (&acc)[4][4], const __nv_bfloat16* a,
+                                           const __nv_bfloat16* wt, int rg, int hf, int lane) {
+    const int r8 = lane & 7, q = lane >> 3;
 #pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-            const int64_t row = r0 + g + 8 * hh;
-            d[hh] = 0.f;
-            if (row < B) {
-                const double tv = target[idx ? idx[row] : row];
-                const float e = y[row] - (float)tv;
-                d[hh] = 2.0f * e / (float)B;
-                if (t == 0) {
-                    dy[row] = d[hh];
-                    lsum += e * e / (float)B;
-                }
-            }
+    for (int kk = 0; kk < KSTEPS; ++kk) {
+        uint32_t af[4];
+        ldsm4(af, a + (16 * rg + (q & 1) * 8 + r8) * LDA + 16 * kk + (q >> 1) * 8);
+#pragma unroll
+        for (int np = 0; np < 2; ++np) {               // two 8-column tiles per load
+            const int n0 = 32 * hf + 16 * np;
+            uint32_t b[4];
+            if constexpr (TRANS)
+                ldsm4t(b, wt + (16 * kk + (q & 1) * 8 + r8) * LDW + n0 + (q >> 1) * 8);
+            else
+                ldsm4(b, wt + (n0 + (q >> 1) * 8 + r8) * LDW + 16 * kk + (q & 1) * 8);
+            mma16816(acc[2 * np], af, b[0], b[1]);
+            mma16816(acc[2 * np + 1], af, b[2], b[3]);
         }
-        // dz3 = dy w4 * gelu'(z3), in accumulator layout
-        float dz[8][4];
+    }
+}
+
+// acc[4][4] += act^T dz over the tile's rows: features 16 mt .., columns 32 hf ..
+template <int LDA>
+__device__ __forceinline__ void train_wgrad(float (&acc)[4][4], const __nv_bfloat16* act,
+                                            const __nv_bfloat16* dz, int mt, int hf, int lane) {
+    const int r8 = lane & 7, q = lane >> 3;
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt)
+    for (int kk = 0; kk < kTrainRows / 16; ++kk) {
+        uint32_t af[4];
+        ldsm4t(af, act + (16 * kk + (q >> 1) * 8 + r8) * LDA + 16 * mt + (q & 1) * 8);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int hh = q >> 1;
-                const int64_t row = r0 + g + 8 * hh;
-                const int col = 8 * nt + 2 * t + (q & 1);
-                dz[nt][q] = row < B ? d[hh] * s.w4[col] * gelu_grad(z3[row * kHid + col]) : 0.f;
+        for (int np = 0; np < 2; ++np) {
+            uint32_t b[4];
+            ldsm4t(b, dz + (16 * kk + (q & 1) * 8 + r8) * kLdH + 32 * hf + 16 * np + (q >> 1) * 8);
+            mma16816(acc[2 * np], af, b[0], b[1]);
+            mma16816(acc[2 * np + 1], af, b[2], b[3]);
+        }
+    }
+}
+
+// Partial gradients and loss of the mean squared error over the CTA's tiles of 64 batch rows, in
+// part[blockIdx.x * kPartStride ..] (packed as the parameters, then the loss). Batch row r is
+// row idx[r] (or r) of X and target. vec: X is 16-byte aligned (else 4-byte loads).
+__global__ void __launch_bounds__(kTrainThreads)
+    k_mlp_train(const __nv_bfloat16* __restrict__ X, const double* __restrict__ target,
+                const int* __restrict__ idx, int64_t B, const float* __restrict__ P,
+                float* __restrict__ part, bool vec) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    TrainSmem& s = *reinterpret_cast<TrainSmem*>(smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int g = lane >> 2, t = lane & 3, rg = warp & 3, hf = warp >> 2;
+    pdl_wait();                                        // the last step's update of P
+    pdl_allow_next();
+    for (int i = tid; i < kHid * kLd1; i += kTrainThreads) {
+        const int k = i / kHid, o = i - k * kHid;      // coalesced reads, transposed stores
+        s.w1t[o * kLd1 + k] = __float2bfloat16_rn(k < kIn ? P[oW1 + k * kHid + o] : 0.f);
+    }
+    for (int i = tid; i < kHid * kHid; i += kTrainThreads) {
+        const int k = i / kHid, o = i - k * kHid;
+        s.w2t[o * kLdH + k] = __float2bfloat16_rn(P[oW2 + i]);
+        s.w3t[o * kLdH + k] = __float2bfloat16_rn(P[oW3 + i]);
+    }
+    if (tid < kHid) {
+        s.bias[0][tid] = P[ob1 + tid];
+        s.bias[1][tid] = P[ob2 + tid];
+        s.bias[2][tid] = P[ob3 + tid];
+        s.w4[tid] = bf16r(P[ow4 + tid]);
+    }
+    if (tid == 0) s.b4 = P[ob4];
+    float wg[3][4][4] = {};                            // weight gradients of W1, W2, W3
+    float sb[3] = {0.f, 0.f, 0.f}, sw4 = 0.f, sdy = 0.f, lsum = 0.f;
+    const float Bf = (float)B;
+    for (int64_t r0 = (int64_t)blockIdx.x * kTrainRows; r0 < B;
+         r0 += (int64_t)gridDim.x * kTrainRows) {
+        __syncthreads();                               // weights staged; the last tile consumed
+        for (int i = tid; i < kTrainRows * (kInPad / 8); i += kTrainThreads) {
+            const int r = i / (kInPad / 8), c = i - r * (kInPad / 8);
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (r0 + r < B) {
+                const int64_t src = idx ? (int64_t)idx[r0 + r] : r0 + r;
+                const __nv_bfloat16* p = X + src * kInPad + 8 * c;
+                if (vec) v = *reinterpret_cast<const uint4*>(p);
+                else v = make_uint4(ld32(p), ld32(p + 2), ld32(p + 4), ld32(p + 6));
             }
-        const float* zs[2] = {z2, z1};
-        __nv_bfloat16* dzs[3] = {dz3, dz2, dz1};
-        const __nv_bfloat16* wn[2] = {s.w3n, s.w2n};
+            *reinterpret_cast<uint4*>(s.x + r * kLd1 + 8 * c) = v;
+        }
+        if (tid < kTrainRows && r0 + tid < B)
+            s.target[tid] = (float)target[idx ? (int64_t)idx[r0 + tid] : r0 + tid];
+        __syncthreads();
+        float gg[3][4][4];                             // gelu'(z) of the thread's cells
+        float acc[4][4];
 #pragma unroll
-        for (int layer = 0; layer < 3; ++layer) {
-            uint32_t a[4][4];
+        for (int l = 0; l < 3; ++l) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                a[kk][0] = pack_bf16(dz[2 * kk][0], dz[2 * kk][1]);
-                a[kk][1] = pack_bf16(dz[2 * kk][2], dz[2 * kk][3]);
-                a[kk][2] = pack_bf16(dz[2 * kk + 1][0], dz[2 * kk + 1][1]);
-                a[kk][3] = pack_bf16(dz[2 * kk + 1][2], dz[2 * kk + 1][3]);
+            for (int nt = 0; nt < 4; ++nt) {
+                const int c = 32 * hf + 8 * nt + 2 * t;
+                acc[nt][0] = acc[nt][2] = s.bias[l][c];
+                acc[nt][1] = acc[nt][3] = s.bias[l][c + 1];
             }
+            if (l == 0) train_gemm<3, kLd1, kLd1, false>(acc, s.x, s.w1t, rg, hf, lane);
+            else train_gemm<4, kLdH, kLdH, false>(acc, s.h[l - 1], l == 1 ? s.w2t : s.w3t, rg, hf,
+                                                  lane);
+            float yp[2] = {0.f, 0.f};
 #pragma unroll
-            for (int nt = 0; nt < 8; ++nt)
+            for (int nt = 0; nt < 4; ++nt) {
+                const int c = 32 * hf + 8 * nt + 2 * t;
 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
-                    const int64_t row = r0 + g + 8 * hh;
-                    if (row < B) {
-                        const int col = 8 * nt + 2 * t;
-                        dzs[layer][row * kHid + col] = __float2bfloat16_rn(dz[nt][2 * hh]);
-                        dzs[layer][row * kHid + col + 1] = __float2bfloat16_rn(dz[nt][2 * hh + 1]);
-                    }
+                    const float h0 = bf16r(gelu_with_grad(acc[nt][2 * hh], &gg[l][nt][2 * hh]));
+                    const float h1 = bf16r(gelu_with_grad(acc[nt][2 * hh + 1],
+                                                          &gg[l][nt][2 * hh + 1]));
+                    *reinterpret_cast<uint32_t*>(s.h[l] + (16 * rg + g + 8 * hh) * kLdH + c) =
+                        pack_bf16(h0, h1);
+                    if (l == 2) yp[hh] += h0 * s.w4[c] + h1 * s.w4[c + 1];
                 }
-            if (layer == 2) break;
-            float dh[8][4];
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt) dh[nt][0] = dh[nt][1] = dh[nt][2] = dh[nt][3] = 0.f;
-            gemm_rows<4>(dh, a, wn[layer], kLdH, g, t);     // dh = dz W^T
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int64_t row = r0 + g + 8 * (q >> 1);
-                    const int col = 8 * nt + 2 * t + (q & 1);
-                    dz[nt][q] = row < B ? dh[nt][q] * gelu_grad(zs[layer][row * kHid + col]) : 0.f;
-                }
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-    if (lane == 0) atomicAdd(loss, lsum);
-}
-
-// part[cta][m][n] = sum over the CTA's rows of act[row][m] dz[row][n]: one warp per 16
-// activation features, rows in chunks of 16 staged transposed in shared memory. The partials are
-// summed over CTAs in a fixed order by k_reduce_parts, so gradients are bitwise reproducible.
-// act: BF16 rows of width lda (gathered through idx when given), features 0..ma-1.
-__global__ void __launch_bounds__(128)
-    k_mlp_wgrad(const __nv_bfloat16* __restrict__ act, int lda, const int* __restrict__ idx,
-                int ma, const __nv_bfloat16* __restrict__ dz, int64_t B, int64_t rows_per_cta,
-                float* __restrict__ part) {
-    __shared__ __align__(16) __nv_bfloat16 sa[kHid][16 + 8];
-    __shared__ __align__(16) __nv_bfloat16 sd[kHid][16 + 8];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int64_t rb = blockIdx.x * rows_per_cta;
-    const int64_t re = min(B, rb + rows_per_cta);
-    float acc[8][4];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-    for (int64_t r0 = rb; r0 < re; r0 += 16) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < 16 * kHid; i += blockDim.x) {
-            const int rr = i / kHid, f = i % kHid;
-            const int64_t row = r0 + rr;
-            const bool ok = row < re;
-            const int64_t src = ok ? (idx ? (int64_t)idx[row] : row) : 0;
-            sa[f][rr] = (ok && f < ma) ? act[src * lda + f] : __float2bfloat16(0.f);
-            sd[f][rr] = ok ? dz[row * kHid + f] : __float2bfloat16(0.f);
-        }
-        __syncthreads();
-        if (16 * warp < ma) {
-            uint32_t a[4];
-            a[0] = ld32(&sa[16 * warp + g][2 * t]);
-            a[1] = ld32(&sa[16 * warp + g + 8][2 * t]);
-            a[2] = ld32(&sa[16 * warp + g][2 * t + 8]);
-            a[3] = ld32(&sa[16 * warp + g + 8][2 * t + 8]);
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt)
-                mma16816(acc[nt], a, ld32(&sd[8 * nt + g][2 * t]), ld32(&sd[8 * nt + g][2 * t + 8]));
-        }
-    }
-    if (16 * warp < ma) {
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int m = 16 * warp + g + 8 * (q >> 1);
-                const int n = 8 * nt + 2 * t + (q & 1);
-                if (m < ma) part[((int64_t)blockIdx.x * ma + m) * kHid + n] = acc[nt][q];
             }
-    }
-}
-
-// bias gradients and the output layer, per block: part[blk][0..319] = (sum dz1, sum dz2,
-// sum dz3, sum h3 dy) per column and sum dy at 256; summed over blocks by k_reduce_parts.
-constexpr int kSmallParts = 4 * kHid + 1;
-constexpr int64_t kRowsPerCta = 1024;          // rows reduced by one weight-gradient CTA
-constexpr int64_t kSmallBlocks = 152 * 4;      // blocks of the small-gradient kernel
-__global__ void k_mlp_small_grads(const __nv_bfloat16* __restrict__ dz1,
-                                  const __nv_bfloat16* __restrict__ dz2,
-                                  const __nv_bfloat16* __restrict__ dz3,
-                                  const __nv_bfloat16* __restrict__ h3,
-                                  const float* __restrict__ dy, int64_t B,
-                                  float* __restrict__ part) {
-    __shared__ float s[4][5][kHid];
-    const int col = threadIdx.x & 63;     // 256 threads: 4 row phases x 64 columns
-    const int ph = threadIdx.x >> 6;
-    float s1 = 0.f, s2 = 0.f, s3 = 0.f, s4 = 0.f, s5 = 0.f;
-    for (int64_t r = blockIdx.x * 4 + ph; r < B; r += (int64_t)gridDim.x * 4) {
-        s1 += __bfloat162float(dz1[r * kHid + col]);
-        s2 += __bfloat162float(dz2[r * kHid + col]);
-        s3 += __bfloat162float(dz3[r * kHid + col]);
-        s4 += __bfloat162float(h3[r * kHid + col]) * dy[r];
-        if (col == 0) s5 += dy[r];
-    }
-    s[ph][0][col] = s1; s[ph][1][col] = s2; s[ph][2][col] = s3; s[ph][3][col] = s4;
-    s[ph][4][col] = s5;
-    __syncthreads();
-    if (ph == 0) {
-        float* p = part + (int64_t)blockIdx.x * kSmallParts;
+            if (l == 2) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            p[q * kHid + col] = ((s[0][q][col] + s[1][q][col]) + s[2][q][col]) + s[3][q][col];
-        if (col == 0) p[4 * kHid] = ((s[0][4][0] + s[1][4][0]) + s[2][4][0]) + s[3][4][0];
+                for (int hh = 0; hh < 2; ++hh) {
+                    yp[hh] += __shfl_xor_sync(0xffffffffu, yp[hh], 1);
+                    yp[hh] += __shfl_xor_sync(0xffffffffu, yp[hh], 2);
+                    if (t == 0) s.ypart[hf][16 * rg + g + 8 * hh] = yp[hh];
+                }
+            }
+            __syncthreads();
+        }
+        if (tid < kTrainRows) {
+            float d = 0.f;
+            if (r0 + tid < B) {
+                const float e = (s.ypart[0][tid] + s.ypart[1][tid]) + s.b4 - s.target[tid];
+                d = 2.0f * e / Bf;
+                lsum += e * e / Bf;
+            }
+            s.dy[tid] = d;                             // rows past B: zero gradients throughout
+        }
+        __syncthreads();
+#pragma unroll
+        for (int l = 2; l >= 0; --l) {                 // dz of layer l, then dh of the one below
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) {
+                const int c = 32 * hf + 8 * nt + 2 * t;
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) {
+                    const int row = 16 * rg + g + 8 * hh;
+                    float d0, d1;
+                    if (l == 2) {
+                        d0 = s.dy[row] * s.w4[c] * gg[l][nt][2 * hh];
+                        d1 = s.dy[row] * s.w4[c + 1] * gg[l][nt][2 * hh + 1];
+                    } else {
+                        d0 = acc[nt][2 * hh] * gg[l][nt][2 * hh];
+                        d1 = acc[nt][2 * hh + 1] * gg[l][nt][2 * hh + 1];
+                    }
+                    *reinterpret_cast<uint32_t*>(s.dz[l] + row * kLdH + c) = pack_bf16(d0, d1);
+                }
+            }
+            __syncthreads();
+            if (l > 0) {
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt)
+                    acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
+                train_gemm<4, kLdH, kLdH, true>(acc, s.dz[l], l == 2 ? s.w3t : s.w2t, rg, hf, lane);
+                train_wgrad<kLdH>(wg[l], s.h[l - 1], s.dz[l], rg, hf, lane);
+            } else if (rg < kInPad / 16) {
+                train_wgrad<kLd1>(wg[0], s.x, s.dz[0], rg, hf, lane);
+            }
+        }
+        const int col = tid & 63, ph = tid >> 6;       // biases and the output layer
+        for (int r = 16 * ph; r < 16 * ph + 16; ++r) {
+#pragma unroll
+            for (int l = 0; l < 3; ++l) sb[l] += __bfloat162float(s.dz[l][r * kLdH + col]);
+            sw4 += __bfloat162float(s.h[2][r * kLdH + col]) * s.dy[r];
+            if (col == 0) sdy += s.dy[r];
+        }
+    }
+    float* out = part + (int64_t)blockIdx.x * kPartStride;
+    const int offs[3] = {oW1, oW2, oW3};
+#pragma unroll
+    for (int l = 0; l < 3; ++l)
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+                const int m = 16 * rg + g + 8 * hh;
+                if (m < (l == 0 ? kIn : kHid))
+                    *reinterpret_cast<float2*>(out + offs[l] + m * kHid + 32 * hf + 8 * nt + 2 * t) =
+                        make_float2(wg[l][nt][2 * hh], wg[l][nt][2 * hh + 1]);
+            }
+    {
+        const int col = tid & 63, ph = tid >> 6;
+        for (int l = 0; l < 3; ++l) s.small[ph][l][col] = sb[l];
+        s.small[ph][3][col] = sw4;
+        if (col == 0) s.small[ph][4][0] = sdy;
+        // rows of the loss live in warps 0 and 1
+        for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+        if (lane == 0 && warp < 2) s.small[0][4][1 + warp] = lsum;
+        __syncthreads();
+        const int goff[4] = {ob1, ob2, ob3, ow4};
+        if (ph == 0)
+            for (int q = 0; q < 4; ++q)
+                out[goff[q] + col] = ((s.small[0][q][col] + s.small[1][q][col]) +
+                                      s.small[2][q][col]) + s.small[3][q][col];
+        if (tid == 0) {
+            out[ob4] = ((s.small[0][4][0] + s.small[1][4][0]) + s.small[2][4][0]) + s.small[3][4][0];
+            out[kParams] = s.small[0][4][1] + s.small[0][4][2];
+        }
     }
 }
 
-// out[i] = sum over blocks b = 0..nblk-1 of part[b * stride + i], in that order
-__global__ void k_reduce_parts(const float* __restrict__ part, int nblk, int64_t stride, int count,
-                               float* __restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count) return;
+// Gradients (and the loss) as the sums of the CTAs' partials, in a fixed order (so bitwise
+// reproducible): slice k of 8 adds partials k, k + 8, ..., then the slices are added in order. With
+// apply set, one Adam step on the FP32 master parameters follows.
+struct AdamStep {
+    int apply = 0;
+    float lr = 0.f, b1 = 0.f, b2 = 0.f, ob1 = 0.f, ob2 = 0.f, eps = 0.f, c1 = 1.f, c2 = 1.f;
+};
+constexpr int kUpdSlices = 8;
+__global__ void __launch_bounds__(32 * kUpdSlices)
+    k_mlp_update(const float* __restrict__ part, int nparts, float* __restrict__ grad,
+                 float* __restrict__ loss, float* __restrict__ P, float* __restrict__ m,
+                 float* __restrict__ v, const AdamStep ad) {
+    __shared__ float sum[kUpdSlices][32];
+    const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;              // < kPartStride
+    pdl_wait();                                        // the partials
+    pdl_allow_next();
     float acc = 0.f;
-    for (int b = 0; b < nblk; ++b) acc += part[(int64_t)b * stride + i];
-    out[i] = acc;
-}
-
-// ob1 = 1 - b1 and ob2 = 1 - b2 are formed in FP64 by the caller: 1.f - 0.999f in FP32 is
-// 1.3e-5 away from 0.001.
-__global__ void k_adam(float* __restrict__ P, float* __restrict__ m, float* __restrict__ v,
-                       const float* __restrict__ g, int n, float lr, float b1, float b2,
-                       float ob1, float ob2, float eps, float c1, float c2) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + ob1 * gi;
-    const float vi = b2 * v[i] + ob2 * (gi * gi);
+#pragma unroll 8
+    for (int b = k; b < nparts; b += kUpdSlices) acc += part[(int64_t)b * kPartStride + i];
+    sum[k][lane] = acc;
+    __syncthreads();
+    if (k != 0 || i > kParams) return;
+    float g = sum[0][lane];
+#pragma unroll
+    for (int q = 1; q < kUpdSlices; ++q) g += sum[q][lane];
+    if (i == kParams) {
+        *loss = g;
+        return;
+    }
+    grad[i] = g;
+    if (!ad.apply) return;
+    const float mi = ad.b1 * m[i] + ad.ob1 * g;
+    const float vi = ad.b2 * v[i] + ad.ob2 * (g * g);
     m[i] = mi;
     v[i] = vi;
-    P[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    P[i] -= ad.lr * (mi / ad.c1) / (sqrtf(vi / ad.c2) + ad.eps);
 }
 
 int nb(int64_t n, int t, int cap = 152 * 16) {
@@ -639,46 +699,28 @@ struct Mlp {
     float* grad = nullptr;
     float* loss = nullptr;
     int64_t step = 0;
-    // training scratch (grown on demand)
-    int64_t cap = 0;
-    float *y = nullptr, *dy = nullptr, *z1 = nullptr, *z2 = nullptr, *z3 = nullptr;
-    __nv_bfloat16 *h1 = nullptr, *h2 = nullptr, *h3 = nullptr;
-    __nv_bfloat16 *d1 = nullptr, *d2 = nullptr, *d3 = nullptr;
-    float* part = nullptr;       // per-CTA gradient partials
+    float* part = nullptr;       // per-CTA partial gradients of a training step (first use)
+    int parts = 0;               // CTAs it has room for
 };
 
 namespace {
 
-void free_mlp_scratch(Mlp* q) {
-    void* ps[] = {q->y, q->dy, q->z1, q->z2, q->z3, q->h1, q->h2, q->h3, q->d1, q->d2, q->d3,
-                  q->part};
-    for (void* p : ps)
-        if (p) cudaFree(p);
-    q->y = q->dy = q->z1 = q->z2 = q->z3 = nullptr;
-    q->h1 = q->h2 = q->h3 = q->d1 = q->d2 = q->d3 = nullptr;
-    q->part = nullptr;
-    q->cap = 0;
+// CTAs of a training step on this device: two per SM, at most one per 64 rows
+ftcg_status_t train_ctas(int64_t B, int* out) {
+    int dev = 0, sms = 0;
+    FTCG_CK(cudaGetDevice(&dev));
+    FTCG_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    *out = (int)std::min<int64_t>((B + kTrainRows - 1) / kTrainRows, 2 * (int64_t)sms);
+    return FTCG_SUCCESS;
 }
 
-ftcg_status_t ensure_scratch(Mlp* q, int64_t B) {
-    if (B <= q->cap) return FTCG_SUCCESS;
-    free_mlp_scratch(q);
-    const size_t nf = (size_t)B * kHid;
-    FTCG_CK(cudaMalloc(&q->y, B * sizeof(float)));
-    FTCG_CK(cudaMalloc(&q->dy, B * sizeof(float)));
-    FTCG_CK(cudaMalloc(&q->z1, nf * sizeof(float)));
-    FTCG_CK(cudaMalloc(&q->z2, nf * sizeof(float)));
-    FTCG_CK(cudaMalloc(&q->z3, nf * sizeof(float)));
-    FTCG_CK(cudaMalloc(&q->h1, nf * 2));
-    FTCG_CK(cudaMalloc(&q->h2, nf * 2));
-    FTCG_CK(cudaMalloc(&q->h3, nf * 2));
-    FTCG_CK(cudaMalloc(&q->d1, nf * 2));
-    FTCG_CK(cudaMalloc(&q->d2, nf * 2));
-    FTCG_CK(cudaMalloc(&q->d3, nf * 2));
-    const int64_t nwb = (B + kRowsPerCta - 1) / kRowsPerCta;
-    const int64_t nsb = std::min<int64_t>((B + 3) / 4, kSmallBlocks);
-    FTCG_CK(cudaMalloc(&q->part, (size_t)std::max<int64_t>(nwb * kHid * kHid, nsb * kSmallParts) * sizeof(float)));
-    q->cap = B;
+ftcg_status_t ensure_parts(Mlp* q, int ctas) {
+    if (ctas <= q->parts) return FTCG_SUCCESS;
+    if (q->part) FTCG_CK(cudaFree(q->part));
+    q->part = nullptr;
+    q->parts = 0;
+    FTCG_CK(cudaMalloc(&q->part, (size_t)ctas * kPartStride * sizeof(float)));
+    q->parts = ctas;
     return FTCG_SUCCESS;
 }
 
@@ -687,58 +729,29 @@ ftcg_status_t mlp_fail(const char* m) {
     return FTCG_ERR_INVALID_VALUE;
 }
 
-size_t fwd_smem() { return sizeof(MlpSmem); }
-
-ftcg_status_t launch_forward(Mlp* q, const __nv_bfloat16* X, const int* idx, int64_t M, bool train,
-                             double* alpha, cudaStream_t s) {
-    const size_t sm = fwd_smem();
+ftcg_status_t launch_forward(Mlp* q, const __nv_bfloat16* X, int64_t M, double* alpha,
+                             cudaStream_t s) {
+    const size_t sm = sizeof(MlpSmem);
     const int blocks = nb((M + 63) / 64, 1, 152 * 8);
-    if (train) {
-        FTCG_CK(cudaFuncSetAttribute(k_mlp_forward<true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        k_mlp_forward<true><<<blocks, 128, sm, s>>>(X, idx, M, q->P, q->y, nullptr, q->z1, q->z2,
-                                                    q->z3, q->h1, q->h2, q->h3);
-    } else {
-        FTCG_CK(cudaFuncSetAttribute(k_mlp_forward<false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        k_mlp_forward<false><<<blocks, 128, sm, s>>>(X, idx, M, q->P, nullptr, alpha, nullptr,
-                                                     nullptr, nullptr, nullptr, nullptr, nullptr);
-    }
+    FTCG_CK(cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sm));
+    k_mlp_forward<<<blocks, 128, sm, s>>>(X, M, q->P, alpha);
     FTCG_CK(cudaGetLastError());
     return FTCG_SUCCESS;
 }
 
-// forward + backward + gradients of one batch into q->grad (zeroed first); loss into q->loss
-ftcg_status_t batch_grads(Mlp* q, const __nv_bfloat16* X, const double* target, const int* idx,
-                          int64_t B, cudaStream_t s) {
-    FTCG_TRY(ensure_scratch(q, B));
-    FTCG_CK(cudaMemsetAsync(q->grad, 0, kParams * sizeof(float), s));
-    FTCG_CK(cudaMemsetAsync(q->loss, 0, sizeof(float), s));
-    FTCG_TRY(launch_forward(q, X, idx, B, true, nullptr, s));
-    const size_t sm = fwd_smem();
-    FTCG_CK(cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    k_mlp_backward<<<nb((B + 63) / 64, 1, 152 * 8), 128, sm, s>>>(
-        target, idx, B, q->P, q->y, q->z1, q->z2, q->z3, q->dy, q->d1, q->d2, q->d3, q->loss);
-    const int wb = (int)((B + kRowsPerCta - 1) / kRowsPerCta);
-    const __nv_bfloat16* acts[3] = {X, q->h1, q->h2};
-    const __nv_bfloat16* dzs[3] = {q->d1, q->d2, q->d3};
-    const int ldas[3] = {kInPad, kHid, kHid};
-    const int mas[3] = {kIn, kHid, kHid};
-    const int offs[3] = {oW1, oW2, oW3};
-    for (int l = 0; l < 3; ++l) {
-        k_mlp_wgrad<<<wb, 128, 0, s>>>(acts[l], ldas[l], l == 0 ? idx : nullptr, mas[l], dzs[l], B,
-                                       kRowsPerCta, q->part);
-        const int cnt = mas[l] * kHid;
-        k_reduce_parts<<<(cnt + 255) / 256, 256, 0, s>>>(q->part, wb, cnt, cnt, q->grad + offs[l]);
-    }
-    const int sb = (int)std::min<int64_t>((B + 3) / 4, kSmallBlocks);
-    k_mlp_small_grads<<<sb, 256, 0, s>>>(q->d1, q->d2, q->d3, q->h3, q->dy, B, q->part);
-    // the groups b1, b2, b3, w4 and b4 go to their places in the packed gradient
-    const int goff[5] = {ob1, ob2, ob3, ow4, ob4};
-    for (int gi = 0; gi < 5; ++gi)
-        k_reduce_parts<<<1, 64, 0, s>>>(q->part + gi * kHid, sb, kSmallParts, gi < 4 ? kHid : 1,
-                                        q->grad + goff[gi]);
-    FTCG_CK(cudaGetLastError());
+// gradients of one batch into q->grad and its loss into q->loss, then (ad.apply) an Adam step
+ftcg_status_t train_batch(Mlp* q, const __nv_bfloat16* X, const double* target, const int* idx,
+                          int64_t B, const AdamStep& ad, cudaStream_t s) {
+    int ctas = 0;
+    FTCG_TRY(train_ctas(B, &ctas));
+    FTCG_TRY(ensure_parts(q, ctas));
+    const size_t sm = sizeof(TrainSmem);
+    FTCG_CK(cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    FTCG_CK(launch_pdl(k_mlp_train, dim3(ctas), dim3(kTrainThreads), sm, s, X, target, idx, B,
+                       (const float*)q->P, q->part, (reinterpret_cast<uintptr_t>(X) & 15) == 0));
+    FTCG_CK(launch_pdl(k_mlp_update, dim3(kPartStride / 32), dim3(32 * kUpdSlices), 0, s,
+                       (const float*)q->part, ctas, q->grad, q->loss, q->P, q->m, q->v, ad));
     return FTCG_SUCCESS;
 }
 
@@ -1001,8 +1014,8 @@ ftcg_status_t ftcg_mlp_predict(ftcg_mlp_t mlp, const void* d_features, int64_t M
         return mlp_fail("ftcg_mlp_predict: bad arguments");
     if (M == 0) return FTCG_SUCCESS;
     Mlp* q = reinterpret_cast<Mlp*>(mlp);
-    return launch_forward(q, reinterpret_cast<const __nv_bfloat16*>(d_features), nullptr, M, false,
-                          d_alpha_out, reinterpret_cast<cudaStream_t>(stream));
+    return launch_forward(q, reinterpret_cast<const __nv_bfloat16*>(d_features), M, d_alpha_out,
+                          reinterpret_cast<cudaStream_t>(stream));
     FTCG_API_END
 }
 
@@ -1014,8 +1027,8 @@ ftcg_status_t ftcg_mlp_grads(ftcg_mlp_t mlp, const void* d_features, const doubl
     if (!mlp || B <= 0 || !d_features || !d_target) return mlp_fail("ftcg_mlp_grads: bad arguments");
     Mlp* q = reinterpret_cast<Mlp*>(mlp);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    FTCG_TRY(batch_grads(q, reinterpret_cast<const __nv_bfloat16*>(d_features), d_target, d_index,
-                         B, s));
+    FTCG_TRY(train_batch(q, reinterpret_cast<const __nv_bfloat16*>(d_features), d_target, d_index,
+                         B, AdamStep{}, s));
     if (h_grads)
         FTCG_CK(cudaMemcpyAsync(h_grads, q->grad, kParams * sizeof(float), cudaMemcpyDeviceToHost, s));
     if (h_loss) FTCG_CK(cudaMemcpyAsync(h_loss, q->loss, sizeof(float), cudaMemcpyDeviceToHost, s));
@@ -1033,16 +1046,13 @@ ftcg_status_t ftcg_mlp_train_step(ftcg_mlp_t mlp, const void* d_features, const 
         return mlp_fail("ftcg_mlp_train_step: bad arguments");
     Mlp* q = reinterpret_cast<Mlp*>(mlp);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    FTCG_TRY(batch_grads(q, reinterpret_cast<const __nv_bfloat16*>(d_features), d_target, d_index,
-                         B, s));
+    // 1 - beta is formed in FP64: 1.f - 0.999f in FP32 is 1.3e-5 away from 0.001
+    const double b1 = 0.9, b2 = 0.999, n = (double)(q->step + 1);
+    const AdamStep ad{1, lr, (float)b1, (float)b2, (float)(1.0 - b1), (float)(1.0 - b2), 1e-8f,
+                      (float)(1.0 - std::pow(b1, n)), (float)(1.0 - std::pow(b2, n))};
+    FTCG_TRY(train_batch(q, reinterpret_cast<const __nv_bfloat16*>(d_features), d_target, d_index,
+                         B, ad, s));
     q->step += 1;
-    const double b1 = 0.9, b2 = 0.999;
-    const float c1 = (float)(1.0 - std::pow(b1, (double)q->step));
-    const float c2 = (float)(1.0 - std::pow(b2, (double)q->step));
-    k_adam<<<(kParams + 255) / 256, 256, 0, s>>>(q->P, q->m, q->v, q->grad, kParams, lr,
-                                                 (float)b1, (float)b2, (float)(1.0 - b1),
-                                                 (float)(1.0 - b2), 1e-8f, c1, c2);
-    FTCG_CK(cudaGetLastError());
     if (h_loss) {
         FTCG_CK(cudaMemcpyAsync(h_loss, q->loss, sizeof(float), cudaMemcpyDeviceToHost, s));
         FTCG_CK(cudaStreamSynchronize(s));
@@ -1057,7 +1067,7 @@ ftcg_status_t ftcg_mlp_destroy(ftcg_mlp_t mlp) {
     if (!mlp) return FTCG_SUCCESS;
     Mlp* q = reinterpret_cast<Mlp*>(mlp);
     cudaDeviceSynchronize();
-    free_mlp_scratch(q);
+    cudaFree(q->part);
     cudaFree(q->P);
     cudaFree(q->m);
     cudaFree(q->v);
