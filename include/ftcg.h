@@ -147,7 +147,8 @@ ftcg_status_t ftcg_plan_info(ftcg_plan_t plan, ftcg_plan_info_t* info);
  *     S_k = sum_j F_N(lambda_jx - lambda_kx) F_N(lambda_jy - lambda_ky),
  *     F_N(d) = sin^2(pi d) / (N^2 sin^2(pi d / N))   (normalised Fejer kernel),
  * i.e. the column-wise least-squares optimum of || T D - I ||_F with T the data-frame Gram matrix
- * on the N x N pixel lattice. Computed in FP64 on the device by the lag route: a gridded adjoint
+ * on the N x N pixel lattice. Computed on the device by the lag route, in FP64 or in FP32 pairs and
+ * 64-bit integers where the window's truncation is larger than their rounding (same error): a gridded adjoint
  * of unit strengths at 2 lambda on a 2N lattice, a product with c(d) = prod (N - |d_i|) / N^2, and
  * a gridded forward transform at 2 lambda (window width opts.weight_width).
  * The weights are installed in the plan (used by every later ftcg_adjoint) and, if d_alpha_out is

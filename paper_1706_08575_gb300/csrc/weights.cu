@@ -22,6 +22,10 @@
 // and the x transforms only over the N rows m_y = 0..N-1 where c is non-zero. W1 stores each
 // sample's 2 w window values and its tap origins so that W3 reads them instead of evaluating
 // them again.
+//
+// This FP64 route serves lag grids above 8192 and windows whose truncation is below what two-float
+// arithmetic resolves (weight_width > 12, large sigma); weights_split.cu takes the others (4.97 ms
+// against about 1.1 on the large ping) and has the rule (split_lag_side).
 
 #include <cuda_runtime.h>
 
@@ -418,6 +422,7 @@ void window_poly(int W, double beta, PolyCoef* out) {
 
 ftcg_status_t compute_weights(Plan& p, double* d_alpha_out, cudaStream_t s) {
     if (p.M == 0) return FTCG_SUCCESS;
+    if (split_lag_side(p) > 0) return compute_weights_split(p, d_alpha_out, s);
     const int Wa = p.opts.weight_width > 0 ? p.opts.weight_width : 12;
     const int N2 = 2 * p.N;
     const int G2 = 2 * p.G;                      // sigma * (2N)
