@@ -432,7 +432,7 @@ ftcg_status_t ftcg_adjoint_small_noalloc(const double* d_lambda, const void* d_v
  * values only) and spread tau with unit weights (ftcg_weights / ftcg_set_weights remove the
  * band again). d_coef_out: NULL or device M x (2r - 1) complex128, row k holding column k of C at
  * rows k - r + 1 .. k + r - 1 (zero outside 0..M-1).
- * Limits: 1 <= r <= 12; M <= 8192 (the construction costs O(M^2 r) FP64 work and 16 M^2 bytes
+ * Limits: 1 <= r <= 12; M <= 8192 (the construction costs O(M^2 r) FP64 work and 8 M^2 bytes
  * of temporary device memory), NOT_SUPPORTED above; FP32 plans only. Synchronises.
  * Errors: NUMERIC if some column's band system is not positive definite (rank-deficient band;
  * that column's coefficients are set to zero).
