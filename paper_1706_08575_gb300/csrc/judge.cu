@@ -14,8 +14,9 @@
 // A lag d = lambda_j - lambda_k is then the exact integer n_j - n_k, wrapped into [-N/2, N/2], plus
 // the FP32 difference f_j - f_k: its absolute error is a few 1e-8 at any distance, and F_N is
 // smooth on that scale (near d = 0 both sines of the quotient carry the same relative error).
-// sin(pi d) = +-sin(pi (f_j - f_k)) since the integer part only flips the sign; the term is then
-// (sin(pi df) / (N sin(pi d / N)))^2 in FP32, a few ulps. Each thread sums its terms in FP32 with
+// sin(pi d) = +-sin(pi (f_j - f_k)) since the integer part only flips the sign; a term is then
+// the square of sin(pi df_x) sin(pi df_y) / (N^2 sin(pi d_x / N) sin(pi d_y / N)) in FP32, a few
+// ulps, with the sines as polynomials on [-1/2, 1/2]. Each thread sums its terms in FP32 with
 // Kahan compensation; the threads' sums are combined in FP64. Samples with a non-finite or huge
 // coordinate are left out of the sums (as the gridding leaves them out), and a judged sample of
 // that kind gets S = NaN, which the verdict skips.
@@ -32,81 +33,113 @@ namespace ftcg {
 namespace {
 
 constexpr int kJudgeThreads = 256;
-constexpr int kJudgeSkip = INT32_MIN;      // n of a sample left out of the sums
+constexpr float kJudgeSkip = 1e30f;        // n of a sample left out of the sums
+constexpr int kJudgeCols = 4;              // judged samples per block
 
-// Per sample {n_x, n_y, f_x, f_y} (the fractions as FP32 bits): lambda mod N = n + f.
+// Per sample {n_x, n_y, f_x, f_y}: lambda mod N = n + f, n an integer (|n| <= N / 2, exact in FP32).
 __global__ void k_judge_prep(const double* __restrict__ lam, int64_t M, int N,
-                             int4* __restrict__ pts) {
+                             float4* __restrict__ pts) {
     const double invN = 1.0 / N;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < M;
          i += (int64_t)gridDim.x * blockDim.x) {
-        int n[2];
-        float f[2];
+        float n[2], f[2];
         bool ok = true;
         for (int a = 0; a < 2; ++a) {
             const double x = lam[2 * i + a];
             ok = ok && isfinite(x) && fabs(x) < 1099511627776.0;     // 2^40
             const double r = ok ? x - N * rint(x * invN) : 0.0;      // |r| <= N/2 (+ rounding)
             const double q = rint(r);
-            n[a] = (int)q;
+            n[a] = (float)q;
             f[a] = (float)(r - q);
         }
-        pts[i] = ok ? make_int4(n[0], n[1], __float_as_int(f[0]), __float_as_int(f[1]))
-                    : make_int4(kJudgeSkip, kJudgeSkip, 0, 0);
+        pts[i] = ok ? make_float4(n[0], n[1], f[0], f[1])
+                    : make_float4(kJudgeSkip, kJudgeSkip, 0.f, 0.f);
     }
 }
 
-// F_N of one axis for the lag dn + df (dn an integer in [-N, N], |df| < 1).
-__device__ __forceinline__ float fejer_axis(int dn, float df, int N, float invN) {
-    if (dn > N / 2) dn -= N;
-    else if (dn < -(N / 2)) dn += N;
-    float dr = (float)dn + df;
-    if (dr > 0.5f * N) dr -= N;                          // exact (Sterbenz); now |dr| <= N/2
-    else if (dr < -0.5f * N) dr += N;
-    if (dr == 0.0f) return 1.0f;
-    const float sf = sinpif(df);                         // sin(pi d) up to sign
-    const float sq = sinpif(dr * invN);
-    const float r = sf / ((float)N * sq);
-    return r * r;
+// sin(pi x) for |x| <= 1/2: x P(x^2), P interpolating sin(pi x) / x at the five Chebyshev points of
+// x^2 in [0, 1/4] (4e-9 relative); the leading coefficient split so that its rounding drops out
+__device__ __forceinline__ float sin_pi32(float x) {
+    const float t = x * x;
+    float q = fmaf(t, 0.07765591227601387f, -0.5982904112834275f);
+    q = fmaf(t, q, 2.550077386528912f);
+    q = fmaf(t, q, -5.167710076668315f);
+    q = fmaf(t, q, 0.0009676400772034f);           // 3.1415926400772034 - 3.140625
+    return fmaf(x, 3.140625f, x * q);
 }
 
+// One axis of F_N^(1/2) for the lag dn + df (dn an integer, |dn| <= N, |df| <= 1), up to sign:
+// numerator sin(pi df), denominator sin(pi d / N); (1, 1 / N) at lag 0.
+__device__ __forceinline__ void fejer_axis(float dn, float df, float N, float invN, float* num,
+                                           float* den) {
+    if (fabsf(dn) > 0.5f * N) dn -= copysignf(N, dn);
+    float dr = dn + df;
+    if (fabsf(dr) > 0.5f * N) dr -= copysignf(N, dr);    // exact (Sterbenz); now |dr| <= N/2
+    const float magic = 12582912.0f;                     // 1.5 * 2^23: rounds to an integer
+    const float fr = df - ((df + magic) - magic);        // sin(pi df) up to sign, |fr| <= 1/2
+    *num = dr == 0.0f ? 1.0f : sin_pi32(fr);
+    *den = dr == 0.0f ? invN : sin_pi32(dr * invN);
+}
+
+// Block (b, p): the sums over part p of the samples of judged samples 4 b .. 4 b + 3, so that a
+// sample's record is loaded once per four terms and the launch fills the GPU whatever K is. Bound:
+// instruction issue (FP32). One block per judged sample with sinpif and two divisions a term took
+// 625 us for K = 256, M = 211,250 (54 M terms); this 153.
 __global__ void __launch_bounds__(kJudgeThreads)
-    k_fejer_sums(const int4* __restrict__ pts, int64_t M, int N, int K, double* __restrict__ S) {
-    const int64_t k = ((int64_t)blockIdx.x * 2 + 1) * M / (2 * (int64_t)K);
-    const int4 pk = pts[k];
-    if (pk.x == kJudgeSkip) {
-        if (threadIdx.x == 0) S[blockIdx.x] = __longlong_as_double(0x7ff8000000000000LL);
-        return;
+    k_fejer_sums(const float4* __restrict__ pts, int64_t M, int N, int K, int64_t per,
+                 double* __restrict__ part) {
+    float4 pk[kJudgeCols];
+    float s[kJudgeCols], c[kJudgeCols];                  // Kahan sums and their compensations
+#pragma unroll
+    for (int i = 0; i < kJudgeCols; ++i) {
+        const int64_t k = min(K - 1, (int)blockIdx.x * kJudgeCols + i);
+        pk[i] = pts[(k * 2 + 1) * M / (2 * (int64_t)K)];
+        s[i] = c[i] = 0.0f;
     }
-    const float fkx = __int_as_float(pk.z), fky = __int_as_float(pk.w);
-    const float invN = 1.0f / N;
-    float s = 0.0f, c = 0.0f;                            // Kahan sum and its compensation
-    for (int64_t j = threadIdx.x; j < M; j += kJudgeThreads) {
-        const int4 q = pts[j];
+    const float Nf = (float)N, invN = 1.0f / Nf, invN2 = invN * invN;
+    const int64_t j1 = min(M, (blockIdx.y + 1) * per);
+    for (int64_t j = blockIdx.y * per + threadIdx.x; j < j1; j += kJudgeThreads) {
+        const float4 q = pts[j];
         if (q.x == kJudgeSkip) continue;
-        const float t = fejer_axis(q.x - pk.x, __int_as_float(q.z) - fkx, N, invN) *
-                        fejer_axis(q.y - pk.y, __int_as_float(q.w) - fky, N, invN);
-        const float y = t - c;
-        const float u = s + y;
-        c = (u - s) - y;
-        s = u;
+#pragma unroll
+        for (int i = 0; i < kJudgeCols; ++i) {
+            float nx, dx, ny, dy;
+            fejer_axis(q.x - pk[i].x, q.z - pk[i].z, Nf, invN, &nx, &dx);
+            fejer_axis(q.y - pk[i].y, q.w - pk[i].w, Nf, invN, &ny, &dy);
+            const float r = (nx * ny) * invN2 / (dx * dy);
+            const float y = fmaf(r, r, -c[i]);
+            const float u = s[i] + y;
+            c[i] = (u - s[i]) - y;
+            s[i] = u;
+        }
     }
-    double acc = (double)s - (double)c;
-    __shared__ double part[kJudgeThreads / 32];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+    __shared__ double sum[kJudgeCols][kJudgeThreads / 32];
+#pragma unroll
+    for (int i = 0; i < kJudgeCols; ++i) {
+        double acc = (double)s[i] - (double)c[i];
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if ((threadIdx.x & 31) == 0) sum[i][threadIdx.x >> 5] = acc;
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    const int i = threadIdx.x, k = blockIdx.x * kJudgeCols + i;
+    if (i < kJudgeCols && k < K) {
         double t = 0.0;
-        for (int w = 0; w < kJudgeThreads / 32; ++w) t += part[w];
-        S[blockIdx.x] = t;
+        for (int w = 0; w < kJudgeThreads / 32; ++w) t += sum[i][w];
+        part[(int64_t)blockIdx.y * K + k] = t;
     }
 }
 
-__global__ void k_gather_alpha(const double* __restrict__ alpha, int64_t M, int K,
-                               double* __restrict__ out) {
+// S_k from its parts, in order (NaN for a judged sample that is left out), and alpha_pred there
+__global__ void k_judge_finish(const double* __restrict__ part, int parts,
+                               const float4* __restrict__ pts, const double* __restrict__ alpha,
+                               int64_t M, int K, double* __restrict__ S, double* __restrict__ a) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < K) out[i] = alpha[((int64_t)i * 2 + 1) * M / (2 * (int64_t)K)];
+    if (i >= K) return;
+    const int64_t j = ((int64_t)i * 2 + 1) * M / (2 * (int64_t)K);
+    double t = 0.0;
+    for (int p = 0; p < parts; ++p) t += part[(int64_t)p * K + i];
+    S[i] = pts[j].x == kJudgeSkip ? __longlong_as_double(0x7ff8000000000000LL) : t;
+    a[i] = alpha[j];
 }
 
 __global__ void k_scale_alpha(const double* __restrict__ a, int64_t M, double s,
@@ -122,13 +155,29 @@ __global__ void k_scale_alpha(const double* __restrict__ a, int64_t M, double s,
 // at the same samples.
 ftcg_status_t judge_launch(const Plan& p, const double* d_alpha, int K, double* d_S,
                            double* d_a, cudaStream_t s) {
-    int4* pts = nullptr;
-    FTCG_CK(pool_malloc(&pts, (size_t)p.M * sizeof(int4), s));
+    // parts: about eight blocks per SM, at least 1024 samples each (and a whole number of strides)
+    const int kb = (K + kJudgeCols - 1) / kJudgeCols;
+    int dev = 0, sms = 0;
+    FTCG_CK(cudaGetDevice(&dev));
+    FTCG_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int64_t want = std::max<int64_t>(1, (8 * (int64_t)sms + kb - 1) / kb);
+    int64_t per = std::max<int64_t>(1024, (p.M + want - 1) / want);
+    per = (per + kJudgeThreads - 1) / kJudgeThreads * kJudgeThreads;
+    const int parts = (int)((p.M + per - 1) / per);
+    float4* pts = nullptr;
+    double* part = nullptr;
+    FTCG_CK(pool_malloc(&pts, (size_t)p.M * sizeof(float4), s));
+    const cudaError_t got = pool_malloc(&part, (size_t)parts * K * sizeof(double), s);
+    if (got != cudaSuccess) {
+        pool_free(pts, s);
+        FTCG_CK(got);
+    }
     const int64_t b = std::min<int64_t>((p.M + 255) / 256, 152 * 8);
     k_judge_prep<<<(unsigned)std::max<int64_t>(1, b), 256, 0, s>>>(p.lambda, p.M, p.N, pts);
-    k_fejer_sums<<<K, kJudgeThreads, 0, s>>>(pts, p.M, p.N, K, d_S);
-    k_gather_alpha<<<(K + 127) / 128, 128, 0, s>>>(d_alpha, p.M, K, d_a);
+    k_fejer_sums<<<dim3(kb, parts), kJudgeThreads, 0, s>>>(pts, p.M, p.N, K, per, part);
+    k_judge_finish<<<(K + 127) / 128, 128, 0, s>>>(part, parts, pts, d_alpha, p.M, K, d_S, d_a);
     const cudaError_t launched = cudaGetLastError();
+    pool_free(part, s);
     FTCG_CK(pool_free(pts, s));
     FTCG_CK(launched);
     return FTCG_SUCCESS;
