@@ -245,6 +245,10 @@ ftcg_status_t adjoint_device(Plan* p, const void* vals, int32_t vdtype, void* im
 
 ftcg_status_t forward_device(Plan* p, const void* img, void* vals, cudaStream_t s) {
     p->last_stream = s;
+    if (p->smem_fft) {
+        FTCG_TRY(exec_smem_fft_forward(p, reinterpret_cast<const float2*>(img), s));
+        return launch_interp(*p, p->grid, reinterpret_cast<float2*>(vals), s);
+    }
     FTCG_TRY(ensure_full_fft(p));
     FTCG_TRY(launch_pad_apod(*p, reinterpret_cast<const float2*>(img), p->grid, s));
     FTCG_CKFFT(cufftSetStream(p->fft, s));

@@ -66,7 +66,60 @@ ftcg_status_t run_smem_fft(const Plan& p, float2* img, cudaStream_t s, cudaEvent
     return FTCG_SUCCESS;
 }
 
+template <int L>
+__global__ void __launch_bounds__(row_threads(L))
+    k_fft_fwd_rows(const float2* __restrict__ img, const unsigned* __restrict__ mask,
+                   const float2* __restrict__ tw, const float2* __restrict__ r2, int N,
+                   float2* __restrict__ grid) {
+    extern __shared__ float2 sm[];
+    pdl_wait();                                // the image, and the last use of the grid
+    pdl_allow_next();
+    fwd_rows_body<L>(img, mask, tw, r2, N, grid, blockIdx.x, sm);
+}
+
+template <int L>
+__global__ void __launch_bounds__(kColThreads, kColMinBlocks)
+    k_fft_fwd_cols(float2* __restrict__ grid, int N, const int* __restrict__ blocks,
+                   const float2* __restrict__ tw) {
+    extern __shared__ float2 sm[];
+    pdl_wait();                                // the row pass is complete
+    pdl_allow_next();
+    fwd_cols_body<L>(grid, N, blocks[blockIdx.x] * kColBlock, tw, sm);
+}
+
+// Large ping (G = 2048, half of the columns occupied), us: zero fill, padding in FP64 and the full
+// cuFFT transform 64; these two passes 24.
+template <int L>
+ftcg_status_t run_smem_fft_forward(const Plan& p, const float2* img, cudaStream_t s) {
+    if (p.n_col_blocks == 0) return FTCG_SUCCESS;
+    const size_t smA = (size_t)kColBlock * col_stride(L) * sizeof(float2);
+    const size_t smB = (size_t)padded_len(L) * sizeof(float2);
+    FTCG_CK(cudaFuncSetAttribute(k_fft_fwd_cols<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smA));
+    FTCG_CK(cudaFuncSetAttribute(k_fft_fwd_rows<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smB));
+    FTCG_CK(launch_pdl(k_fft_fwd_rows<L>, dim3(p.N), dim3(row_threads(L)), smB, s, img,
+                       (const unsigned*)p.col_mask, (const float2*)p.tw, (const float2*)p.deapod2,
+                       p.N, p.grid));
+    FTCG_CK(launch_pdl(k_fft_fwd_cols<L>, dim3(p.n_col_blocks), dim3(kColThreads), smA, s, p.grid,
+                       p.N, (const int*)p.col_blocks, (const float2*)p.tw));
+    return FTCG_SUCCESS;
+}
+
 }  // namespace
+
+ftcg_status_t exec_smem_fft_forward(Plan* p, const float2* img, cudaStream_t s) {
+    switch (p->G) {
+        case 256: return run_smem_fft_forward<256>(*p, img, s);
+        case 512: return run_smem_fft_forward<512>(*p, img, s);
+        case 1024: return run_smem_fft_forward<1024>(*p, img, s);
+        case 2048: return run_smem_fft_forward<2048>(*p, img, s);
+        case 4096: return run_smem_fft_forward<4096>(*p, img, s);
+        default:
+            set_error("internal: no shared-memory FFT for G = %d", p->G);
+            return FTCG_ERR_NOT_SUPPORTED;
+    }
+}
 
 bool smem_fft_supported(int G) {
     return G >= 256 && G <= 4096 && (G & (G - 1)) == 0;

@@ -360,6 +360,54 @@ __device__ __forceinline__ void rows_body(const float2* __restrict__ grid,
     transform<L, 1, NT>(sm, tw, ld, st);
 }
 
+// Forward transform (exponent sign -) of the image, pruned the same way: a transform with sign - is
+// the conjugate of the sign + one of the conjugate, and the grid holds the conjugates between the
+// passes. Row pass: image row iy times the window factors (the product with the FP32 pairs rounded
+// once), zero elsewhere, transformed along x into grid row (iy - N/2) mod L, only in the column
+// blocks that taps reach.
+template <int L>
+__device__ __forceinline__ void fwd_rows_body(const float2* __restrict__ img,
+                                              const unsigned* __restrict__ mask,
+                                              const float2* __restrict__ tw,
+                                              const float2* __restrict__ r2, int N,
+                                              float2* __restrict__ grid, int iy, float2* sm) {
+    constexpr int NT = row_threads(L);
+    const int qy = iy - N / 2 < 0 ? iy - N / 2 + L : iy - N / 2;
+    const float2 ry = r2[iy];
+    const float2* in = img + (int64_t)iy * N;
+    auto ld = [&](int, int kx) {
+        int ix;
+        if (kx < N / 2) ix = kx + N / 2;
+        else if (kx >= L - N / 2) ix = kx - (L - N / 2);
+        else return make_float2(0.f, 0.f);
+        const float2 v = in[ix], rx = r2[ix];
+        const float h = ry.x * rx.x;
+        const float l = fmaf(ry.x, rx.x, -h) + fmaf(ry.x, rx.y, ry.y * rx.x);
+        return make_float2(fmaf(v.x, h, v.x * l), -fmaf(v.y, h, v.y * l));
+    };
+    float2* row = grid + (int64_t)qy * L;
+    auto st = [&](int, int x, float2 h) {
+        const int blk = x / kColBlock;
+        if ((__ldg(mask + (blk >> 5)) >> (blk & 31)) & 1u) row[x] = h;
+    };
+    transform<L, 1, NT>(sm, tw, ld, st);
+}
+
+// Column pass: only the N rows that the row pass wrote are read, all L are written.
+template <int L>
+__device__ __forceinline__ void fwd_cols_body(float2* __restrict__ grid, int N, int x0,
+                                              const float2* __restrict__ tw, float2* sm) {
+    auto ld4 = [&](int c, int y) {
+        if (y >= N / 2 && y < L - N / 2) return make_float4(0.f, 0.f, 0.f, 0.f);
+        return *reinterpret_cast<const float4*>(grid + (int64_t)y * L + x0 + c);
+    };
+    auto st4 = [&](int c, int y, float2 a, float2 b) {
+        *reinterpret_cast<float4*>(grid + (int64_t)y * L + x0 + c) =
+            make_float4(a.x, -a.y, b.x, -b.y);
+    };
+    transform_cols<L, kColBlock, kColThreads>(sm, tw, ld4, st4);
+}
+
 // the stage tables of a transform of length L (see tw_offset), in FP64 rounded to FP32
 template <int L>
 std::vector<float2> stage_twiddles() {

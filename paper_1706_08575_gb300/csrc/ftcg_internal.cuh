@@ -294,6 +294,8 @@ ftcg_status_t build_smem_fft(Plan* p, const std::vector<unsigned char>& occ, cud
 // between the column and the row pass
 ftcg_status_t exec_smem_fft(Plan* p, float2* img, cudaStream_t s, cudaEvent_t mid);
 void release_smem_fft(Plan* p);
+// image (divided by the window transforms) -> grid, forward, in the columns that taps reach
+ftcg_status_t exec_smem_fft_forward(Plan* p, const float2* img, cudaStream_t s);
 ftcg_status_t exec_pruned_inverse(Plan* p, cudaStream_t s);
 void release_pruned_fft(Plan* p);
 

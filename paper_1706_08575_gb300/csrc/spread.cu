@@ -15,6 +15,8 @@
 // grid cell is written exactly once, with no zero-fill. In the halo layout the accumulator also
 // holds the w - 1 overflow rows and columns, which k_halo_add adds to the neighbouring tiles.
 
+#include <algorithm>
+
 #include "spread_window.cuh"
 
 namespace ftcg {
@@ -147,6 +149,88 @@ __global__ void __launch_bounds__(256)
     }
 }
 
+// The same over the plan's tiles: a CTA per chunk samples of a tile holds its cells and the taps' reach in
+// shared memory, four lanes per sample (in the tile's sorted order; samp by sample index); lane q
+// has taps q, q + 4, ... of both axes and sums its columns over the rows. A sample listed in several
+// tiles (duplicate layout) is taken in the tile of its first tap. From global memory, 8 lanes per
+// sample and 8 rows of 64 bytes, the large ping took 165 us, bound by L1 request rate; here 77, bound by
+// shared-memory bank conflicts and the gathers by sample index.
+constexpr int kInterpThreads = 256;
+template <int CPL>
+__global__ void __launch_bounds__(kInterpThreads)
+    k_interp_tiles(const int4* __restrict__ samp, const Entry* __restrict__ ent,
+                   const int* __restrict__ colptr, const int* __restrict__ tile_order, int ncb, int chunk,
+                   const float2* __restrict__ grid, float2* __restrict__ out, int G, int T, int ntx,
+                   int W, Win32 win) {
+    extern __shared__ float2 s_tile[];
+    const int tile = tile_order[blockIdx.x];
+    const int ty = tile / ntx, tx = tile - ty * ntx, X0 = tx * T, Y0 = ty * T;
+    const int side = T + W - 1, ld = side | 1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = threadIdx.x & 3;
+    // part blockIdx.y of the tile's samples
+    const int e0 = colptr[(int64_t)tile * ncb] + (int)blockIdx.y * chunk;
+    const int e1 = min(colptr[(int64_t)(tile + 1) * ncb], e0 + chunk);
+    if (e0 >= e1) return;
+    pdl_wait();                                // the grid is complete
+    // a ragged tile's samples start on its own cells only (G >= 2 w: at most one wrap)
+    const int rows = min(T, G - Y0) + W - 1, cols = min(T, G - X0) + W - 1;
+    for (int r = warp; r < rows; r += kInterpThreads / 32) {
+        int row = Y0 + r;
+        if (row >= G) row -= G;
+        for (int c = lane; c < cols; c += 32) {
+            int col = X0 + c;
+            if (col >= G) col -= G;
+            s_tile[r * ld + c] = grid[(int64_t)row * G + col];
+        }
+    }
+    __syncthreads();
+    for (int b = e0; b < e1; b += kInterpThreads / 4) {
+        const int e = b + threadIdx.x / 4;
+        int j = -1;
+        int4 sm = make_int4(X0, Y0, 0, 0);
+        if (e < e1) {
+            j = (int)(ent[e].packed & kSampleMask);
+            const int4 v = samp[j];
+            if (v.x >= X0 && v.x < X0 + T && v.y >= Y0 && v.y < Y0 + T) sm = v;
+            else j = -1;                       // first tap in another tile
+        }
+        const float dx = __int_as_float(sm.z), dy = __int_as_float(sm.w);
+        float fx[CPL], fy[CPL], re[CPL], im[CPL];
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) {
+            const int l = q + 4 * c;
+            fx[c] = l < W ? win32(dx - (float)l, win) : 0.0f;
+            fy[c] = l < W ? win32(dy - (float)l, win) : 0.0f;
+            re[c] = im[c] = 0.0f;
+        }
+        const float2* g = s_tile + (sm.y - Y0) * ld + (sm.x - X0) + q;
+#pragma unroll
+        for (int r = 0; r < 4 * CPL; ++r) {
+            if (r >= W) break;
+            const float py = __shfl_sync(0xffffffffu, fy[r >> 2], r & 3, 4);
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) {
+                if (q + 4 * c >= W) continue;
+                const float2 h = g[r * ld + 4 * c];
+                re[c] = fmaf(py, h.x, re[c]);
+                im[c] = fmaf(py, h.y, im[c]);
+            }
+        }
+        float sr = 0.0f, si = 0.0f;
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) {
+            sr = fmaf(fx[c], re[c], sr);
+            si = fmaf(fx[c], im[c], si);
+        }
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            sr += __shfl_xor_sync(0xffffffffu, sr, o);
+            si += __shfl_xor_sync(0xffffffffu, si, o);
+        }
+        if (q == 0 && j >= 0) out[j] = make_float2(sr, si);
+    }
+}
+
 // ---- per-entry weights ---------------------------------------------------------------------
 __global__ void k_set_alpha(Entry* __restrict__ ent, int64_t n, const void* __restrict__ alpha,
                             int dtype, bool bf16) {
@@ -233,6 +317,30 @@ ftcg_status_t launch_pad_apod(const Plan& p, const float2* img, float2* grid, cu
 ftcg_status_t launch_interp(const Plan& p, const float2* grid, float2* vals, cudaStream_t s) {
     if (p.M == 0) return FTCG_SUCCESS;
     const Win32 win = win32_of(p.win);
+    const Binning& b = p.bin;
+    // Tiles pay with enough samples to fill the GPU and to amortise loading a tile's cells: from
+    // about 100 k samples and 1/8 sample per cell of the non-empty tiles on. Whole call before and
+    // after, us, w = 8, T = 32 (T = 64): N = 1024, 2.1 M samples 189, 101 (189, 120); 524 k 65, 48
+    // (65, 56); 131 k at 79 per tile 33, 33; N = 256, 200 k 29, 24 (30, 28), 50 k 17, 18 (17, 21);
+    // N = 500 (cuFFT), 180 k 47, 42 (47, 43), 45 k 36, 36 (36, 40).
+    if (p.M >= 98304 && b.n_entries >= (int64_t)b.T * b.T / 8 * b.n_nonempty) {
+        // samples that are in no tile (not finite) read zero
+        if (!b.halo || b.n_entries < p.M)
+            FTCG_CK(cudaMemsetAsync(vals, 0, (size_t)p.M * sizeof(float2), s));
+        const int side = b.T + b.W - 1;
+        const size_t sm = (size_t)side * (side | 1) * sizeof(float2);
+        auto kern = p.w <= 8 ? k_interp_tiles<2> : k_interp_tiles<4>;
+        FTCG_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        // parts of 256 to 1024 samples: eight CTAs per SM where the raster allows it
+        const int chunk =
+            (int)std::min<int64_t>(1024, std::max<int64_t>(256, p.M / (8 * 152) / 64 * 64));
+        const int parts = (b.tile_cnt[b.h_order[0]] + chunk - 1) / chunk;
+        FTCG_CK(launch_pdl(kern, dim3(b.n_nonempty, parts), dim3(kInterpThreads), sm, s,
+                           (const int4*)p.samp, (const Entry*)b.ent, (const int*)b.colptr,
+                           (const int*)b.tile_order, b.ncb, chunk, grid, vals, b.G, b.T, b.ntx,
+                           b.W, win));
+        return FTCG_SUCCESS;
+    }
     if (p.w <= 8) {
         k_interp<8><<<blocks_for(p.M * 8, 256), 256, 0, s>>>(p.samp, p.M, grid, vals, p.G, p.w,
                                                              win);
