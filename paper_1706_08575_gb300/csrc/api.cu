@@ -43,16 +43,13 @@ void release_plan(Plan* p) {
     if (!p) return;
     cudaDeviceSynchronize();
     free_binning(p->bin);
-    if (p->lambda) cudaFree(p->lambda);
-    if (p->samp) cudaFree(p->samp);
-    if (p->deapod) cudaFree(p->deapod);
-    if (p->deapod2) cudaFree(p->deapod2);
-    if (p->grid) cudaFree(p->grid);
-    if (p->status) cudaFree(p->status);
-    if (p->stage_vals) cudaFree(p->stage_vals);
-    if (p->alpha_cur) cudaFree(p->alpha_cur);
+    // pool memory, after the synchronisation above: returned to the pool at once (cudaFree of it
+    // waits and costs several microseconds a buffer)
+    for (void* q : {(void*)p->lambda, (void*)p->samp, (void*)p->deapod, (void*)p->deapod2,
+                    (void*)p->grid, (void*)p->status, p->stage_vals, (void*)p->alpha_cur,
+                    p->stage_img})
+        pool_free(q, nullptr);
     release_band(p);
-    if (p->stage_img) cudaFree(p->stage_img);
     for (int k = 0; k < 2; ++k) {
         if (p->pipe_vals[k]) cudaFree(p->pipe_vals[k]);
         if (p->pipe_up[k]) cudaEventDestroy(p->pipe_up[k]);
@@ -87,15 +84,16 @@ ftcg_status_t make_plan(Plan* p, const double* d_lambda, cudaStream_t s, bool ow
     bytes += (int64_t)p->N * sizeof(float2);
     FTCG_TRY(split_factors(p->deapod, p->deapod2, p->N, s));
     p->bin.det = p->opts.deterministic != 0;
-    FTCG_TRY(build_binning(p->bin, p->lambda, M, p->sigma, p->G, p->opts.tile, p->w,
-                           p->opts.layout == FTCG_LAYOUT_HALO, p->status, p->samp, s, &bytes));
-    if (p->bin.halo && p->opts.spread_kernel != FTCG_SPREAD_WINDOW && p->w <= kMmaMaxW) {
-        double err = 0;
-        if (mma_window_poly(p->w, p->win.beta, p->win.kind, &p->bin.poly, &err))
-            // AUTO (tile side and layout given, so no tuner): the block kernel, the faster one
-            FTCG_TRY(build_chunks(p->bin, s, &bytes,
-                                  p->opts.spread_kernel != FTCG_SPREAD_TENSOR));
-    }
+    // AUTO (tile side and layout given, so no tuner): the block kernel, the faster one
+    double err = 0;
+    const bool halo = p->opts.layout == FTCG_LAYOUT_HALO;
+    const bool tensor = halo && p->opts.spread_kernel != FTCG_SPREAD_WINDOW && p->w <= kMmaMaxW &&
+                        mma_window_poly(p->w, p->win.beta, p->win.kind, &p->bin.poly, &err);
+    const bool column = p->opts.spread_kernel == FTCG_SPREAD_TENSOR;
+    unsigned st = 0;
+    FTCG_TRY(build_binning(p->bin, p->lambda, M, p->sigma, p->G, p->opts.tile, p->w, halo,
+                           tensor && !column, p->status, p->samp, s, &bytes, &st));
+    if (tensor && column) FTCG_TRY(build_column_chunks(p->bin, s, &bytes));
     if (own_grid) {
         FTCG_CK(pool_malloc(&p->grid, (size_t)p->G * p->G * sizeof(float2), s));
         bytes += (int64_t)p->G * p->G * sizeof(float2);
@@ -103,11 +101,9 @@ ftcg_status_t make_plan(Plan* p, const double* d_lambda, cudaStream_t s, bool ow
         FTCG_TRY(build_pruned_fft(p, s, &bytes));
     }
     p->device_bytes = bytes;
-    unsigned st = 0;
-    FTCG_CK(cudaMemcpyAsync(&st, p->status, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-    FTCG_CK(cudaStreamSynchronize(s));
+    if (st & STATUS_NONFINITE_COORD) FTCG_CK(cudaMemsetAsync(p->status, 0, sizeof(unsigned), s));
+    FTCG_CK(cudaStreamSynchronize(s));            // complete on return, whatever stream uses it
     if (st & STATUS_NONFINITE_COORD) {
-        FTCG_CK(cudaMemsetAsync(p->status, 0, sizeof(unsigned), s));
         set_error("ftcg_plan: some coordinates are not finite (or |sigma lambda| >= 2^50); those "
                   "samples are dropped");
         return FTCG_ERR_NUMERIC;

@@ -19,6 +19,9 @@
 
 #include <algorithm>
 #include <cmath>
+#include <map>
+#include <mutex>
+#include <utility>
 #include <vector>
 
 namespace ftcg {
@@ -57,11 +60,11 @@ ftcg_status_t run_smem_fft(const Plan& p, float2* img, cudaStream_t s, cudaEvent
                                  (int)smB));
     if (p.n_col_blocks > 0) {
         FTCG_CK(launch_pdl(k_fft_cols<L>, dim3(p.n_col_blocks), dim3(kColThreads), smA, s,
-                           p.grid, (const int*)p.col_blocks, (const float2*)p.tw));
+                           p.grid, (const int*)p.col_blocks, p.tw));
     }
     if (mid) FTCG_CK(cudaEventRecord(mid, s));
     FTCG_CK(launch_pdl(k_fft_rows_crop<L>, dim3(p.N), dim3(row_threads(L)), smB, s,
-                       (const float2*)p.grid, (const unsigned*)p.col_mask, (const float2*)p.tw,
+                       (const float2*)p.grid, (const unsigned*)p.col_mask, p.tw,
                        (const float2*)p.deapod2, p.N, img));
     return FTCG_SUCCESS;
 }
@@ -99,10 +102,10 @@ ftcg_status_t run_smem_fft_forward(const Plan& p, const float2* img, cudaStream_
     FTCG_CK(cudaFuncSetAttribute(k_fft_fwd_rows<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smB));
     FTCG_CK(launch_pdl(k_fft_fwd_rows<L>, dim3(p.N), dim3(row_threads(L)), smB, s, img,
-                       (const unsigned*)p.col_mask, (const float2*)p.tw, (const float2*)p.deapod2,
+                       (const unsigned*)p.col_mask, p.tw, (const float2*)p.deapod2,
                        p.N, p.grid));
     FTCG_CK(launch_pdl(k_fft_fwd_cols<L>, dim3(p.n_col_blocks), dim3(kColThreads), smA, s, p.grid,
-                       p.N, (const int*)p.col_blocks, (const float2*)p.tw));
+                       p.N, (const int*)p.col_blocks, p.tw));
     return FTCG_SUCCESS;
 }
 
@@ -125,6 +128,42 @@ bool smem_fft_supported(int G) {
     return G >= 256 && G <= 4096 && (G & (G - 1)) == 0;
 }
 
+namespace {
+
+// Stage tables of the five sides, per device, made on first use and kept (60 KB in all): a plan
+// that computes its own spends 30 us in the host's sines and a transfer.
+std::mutex g_tw_mu;
+std::map<std::pair<int, int>, float2*> g_tw;
+
+ftcg_status_t side_twiddles(int G, cudaStream_t s, const float2** out) {
+    int dev = 0;
+    FTCG_CK(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(g_tw_mu);
+    auto it = g_tw.find({dev, G});
+    if (it == g_tw.end()) {
+        std::vector<float2> tw;
+        switch (G) {
+            case 256: tw = stage_twiddles<256>(); break;
+            case 512: tw = stage_twiddles<512>(); break;
+            case 1024: tw = stage_twiddles<1024>(); break;
+            case 2048: tw = stage_twiddles<2048>(); break;
+            default: tw = stage_twiddles<4096>(); break;
+        }
+        float2* d = nullptr;
+        FTCG_CK(cudaMalloc(&d, tw.size() * sizeof(float2)));
+        cudaError_t e = cudaMemcpyAsync(d, tw.data(), tw.size() * sizeof(float2),
+                                        cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // complete before another stream's use
+        if (e != cudaSuccess) cudaFree(d);
+        FTCG_CK(e);
+        it = g_tw.emplace(std::make_pair(dev, G), d).first;
+    }
+    *out = it->second;
+    return FTCG_SUCCESS;
+}
+
+}  // namespace
+
 ftcg_status_t build_smem_fft(Plan* p, const std::vector<unsigned char>& occ, cudaStream_t s,
                              int64_t* bytes) {
     const int G = p->G;
@@ -135,30 +174,17 @@ ftcg_status_t build_smem_fft(Plan* p, const std::vector<unsigned char>& occ, cud
         if (any) blocks.push_back(b);
     }
     p->n_col_blocks = (int)blocks.size();
-    std::vector<unsigned> mask((G / kColBlock + 31) / 32, 0u);
-    for (int b : blocks) mask[b >> 5] |= 1u << (b & 31);
-    FTCG_CK(pool_malloc(&p->col_mask, mask.size() * sizeof(unsigned), s));
-    *bytes += mask.size() * sizeof(unsigned);
-    FTCG_CK(cudaMemcpyAsync(p->col_mask, mask.data(), mask.size() * sizeof(unsigned),
+    const size_t nmask = (G / kColBlock + 31) / 32, nblk = blocks.size();
+    std::vector<int> up(nblk + nmask, 0);               // the blocks, then the mask
+    std::copy(blocks.begin(), blocks.end(), up.begin());
+    for (int b : blocks) up[nblk + (b >> 5)] |= (int)(1u << (b & 31));
+    FTCG_CK(pool_malloc(&p->col_blocks, up.size() * sizeof(int), s));
+    *bytes += up.size() * sizeof(int);
+    p->col_mask = reinterpret_cast<unsigned*>(p->col_blocks + nblk);
+    FTCG_CK(cudaMemcpyAsync(p->col_blocks, up.data(), up.size() * sizeof(int),
                             cudaMemcpyHostToDevice, s));
-    std::vector<float2> tw;
-    switch (G) {
-        case 256: tw = stage_twiddles<256>(); break;
-        case 512: tw = stage_twiddles<512>(); break;
-        case 1024: tw = stage_twiddles<1024>(); break;
-        case 2048: tw = stage_twiddles<2048>(); break;
-        default: tw = stage_twiddles<4096>(); break;
-    }
-    FTCG_CK(pool_malloc(&p->tw, tw.size() * sizeof(float2), s));
-    *bytes += tw.size() * sizeof(float2);
-    FTCG_CK(cudaMemcpyAsync(p->tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice, s));
-    if (!blocks.empty()) {
-        FTCG_CK(pool_malloc(&p->col_blocks, blocks.size() * sizeof(int), s));
-        *bytes += blocks.size() * sizeof(int);
-        FTCG_CK(cudaMemcpyAsync(p->col_blocks, blocks.data(), blocks.size() * sizeof(int),
-                                cudaMemcpyHostToDevice, s));
-    }
-    FTCG_CK(cudaStreamSynchronize(s));          // the host vectors go out of scope
+    FTCG_TRY(side_twiddles(G, s, &p->tw));
+    FTCG_CK(cudaStreamSynchronize(s));          // the host vector goes out of scope
     p->smem_fft = true;
     return FTCG_SUCCESS;
 }
@@ -177,9 +203,7 @@ ftcg_status_t exec_smem_fft(Plan* p, float2* img, cudaStream_t s, cudaEvent_t mi
 }
 
 void release_smem_fft(Plan* p) {
-    if (p->tw) cudaFree(p->tw);
-    if (p->col_blocks) cudaFree(p->col_blocks);
-    if (p->col_mask) cudaFree(p->col_mask);
+    pool_free(p->col_blocks, nullptr);
     p->col_mask = nullptr;
     p->tw = nullptr;
     p->col_blocks = nullptr;

@@ -217,10 +217,10 @@ struct Plan {
     // Shared-memory transforms for power-of-two G (fft_smem.cu): the column blocks that taps
     // reach, and the FP32 twiddle tables of the transform stages.
     bool smem_fft = false;
-    int* col_blocks = nullptr;
+    int* col_blocks = nullptr;          // one allocation with col_mask
     int n_col_blocks = 0;
     unsigned* col_mask = nullptr;       // the same blocks as a bit mask
-    float2* tw = nullptr;
+    const float2* tw = nullptr;         // shared by all plans of the side, not owned
     unsigned* status = nullptr;         // device status word
     // banded FTCG coefficients (band.cu): M x (2 band_r - 1) complex128 and the values buffer
     // tau = C v that the adjoint spreads; band_r = 0 when the diagonal weights are in use
@@ -260,9 +260,10 @@ void release_plan(Plan* p);
 // Launchers (defined in the .cu files)
 // ---------------------------------------------------------------------------------------------
 // plan.cu
+// block_chunks: the block kernel's chunks too; *status: the device status word after the binning
 ftcg_status_t build_binning(Binning& b, const double* d_lambda, int64_t M, double scale,
-                            int G, int T, int W, bool halo, unsigned* d_status, int4* d_samp,
-                            cudaStream_t s, int64_t* bytes);
+                            int G, int T, int W, bool halo, bool block_chunks, unsigned* d_status,
+                            int4* d_samp, cudaStream_t s, int64_t* bytes, unsigned* status);
 void free_binning(Binning& b);
 ftcg_status_t exclusive_scan_i32(const int* d_in, int* d_out, int64_t n, cudaStream_t s);
 // spread.cu
@@ -274,7 +275,14 @@ ftcg_status_t launch_deapod_crop(const Plan& p, const float2* grid, float2* img,
 // spread_mma.cu: the tensor-core spreading path (halo layout, w <= 8)
 // fit the per-tap window polynomials; returns false if their error exceeds the path's bound
 bool mma_window_poly(int W, double beta, int kind, MmaPoly* out, double* max_err);
-ftcg_status_t build_chunks(Binning& b, cudaStream_t s, int64_t* bytes, bool block = false);
+ftcg_status_t build_column_chunks(Binning& b, cudaStream_t s, int64_t* bytes);
+// the block kernel's chunks in two steps: chunks per (tile, 8 x 8 block) from the sort's key starts,
+// their offsets and total (device); after the scatter, from its key ends, the chunks themselves
+ftcg_status_t count_block_chunks(const Binning& b, const int* start, int64_t nkeys,
+                                 const int* d_entries, int* cnt, int* off, int* d_total,
+                                 cudaStream_t s);
+ftcg_status_t finish_block_chunks(Binning& b, const int* end, const int* cnt, const int* off,
+                                  int total, cudaStream_t s, int64_t* bytes);
 void free_chunks(Binning& b);
 ftcg_status_t launch_spread_mma(const Plan& p, const void* vals, bool vbf, float2* grid,
                                 cudaStream_t s, int nt);

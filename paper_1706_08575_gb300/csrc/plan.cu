@@ -9,6 +9,9 @@
 // Entries are ordered by (tile, local first-tap column, local first-tap row) with a counting sort
 // (one wide radix digit: the whole key). Keys are few enough (tiles * (T + w - 1)^2) that one
 // histogram + one exclusive scan + one scatter replace a multi-pass radix sort.
+//
+// The build queues everything it can before its first synchronisation: the host learns all sizes
+// (entries, chunks, samples per tile, occupied columns, status word) from one summary buffer.
 
 #include <algorithm>
 #include <cstdio>
@@ -34,8 +37,9 @@ struct TapOrigin {
 __device__ __forceinline__ TapOrigin tap_origin(double lam, double scale, int W) {
     TapOrigin t;
     double u = __dmul_rn(scale, lam);
-    // |u| < 2^50 keeps ceil() and the int64 arithmetic exact.
-    t.ok = isfinite(u) && fabs(u) < 1125899906842624.0;
+    // finite and |u| < 2^50, which keeps ceil() and the int64 arithmetic exact (from the exponent
+    // bits: FP64 comparisons share the scarce FP64 pipe)
+    t.ok = ((unsigned)__double2hiint(u) & 0x7fffffffu) < (1023u + 50u) << 20;
     if (!t.ok) {
         t.c = 0;
         t.d = 0;
@@ -48,6 +52,8 @@ __device__ __forceinline__ TapOrigin tap_origin(double lam, double scale, int W)
 }
 
 __device__ __forceinline__ int wrap(long long c, int G) {
+    if (c >= -(long long)G && c < 2ll * G)           // the usual case without a 64-bit division
+        return (int)(c < 0 ? c + G : c >= G ? c - G : c);
     long long r = c % G;
     return (int)(r < 0 ? r + G : r);
 }
@@ -135,21 +141,24 @@ __global__ void k_key_sort(const int* __restrict__ cnt, const int* __restrict__ 
     }
 }
 
-__global__ void k_bin_scatter(const double* __restrict__ lam, int64_t M, double scale, int G,
-                              int T, int W, int ntx, int ncb, bool halo,
-                              int* __restrict__ cursor, Entry* __restrict__ ent) {
+// The entries at their sorted places (from the first taps and offsets that k_bin_count stored; in
+// FP64 from the coordinates this took 80 us on the large ping, here 27), and the zeroed ones after
+// the last. cursor: the start offsets of the keys, their ends afterwards.
+__global__ void k_bin_scatter(const int4* __restrict__ samp, int64_t M, int G, int T, int W,
+                              int ntx, int ncb, bool halo, int* __restrict__ cursor,
+                              const int* __restrict__ total, Entry* __restrict__ ent) {
+    if (blockIdx.x == 0 && threadIdx.x < kEntryPad)
+        ent[*total + threadIdx.x] = Entry{0.f, 0.f, 0u, 0u};
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < M;
          j += (int64_t)gridDim.x * blockDim.x) {
-        TapOrigin ox = tap_origin(lam[2 * j], scale, W);
-        TapOrigin oy = tap_origin(lam[2 * j + 1], scale, W);
-        if (!ox.ok || !oy.ok) continue;
-        int cxw = wrap(ox.c, G), cyw = wrap(oy.c, G);
+        const int4 sm = samp[j];
+        if (sm.x < 0) continue;
         Entry e;
-        e.dx = __double2float_rn(ox.d);
-        e.dy = __double2float_rn(oy.d);
+        e.dx = __int_as_float(sm.z);
+        e.dy = __int_as_float(sm.w);
         e.alpha = __float_as_uint(1.0f);
-        Runs rx = axis_runs(cxw, G, T, W, halo);
-        Runs ry = axis_runs(cyw, G, T, W, halo);
+        Runs rx = axis_runs(sm.x, G, T, W, halo);
+        Runs ry = axis_runs(sm.y, G, T, W, halo);
         for (int a = 0; a < ry.n; ++a)
             for (int b = 0; b < rx.n; ++b) {
                 int64_t tile = (int64_t)ry.tile[a] * ntx + rx.tile[b];
@@ -161,12 +170,36 @@ __global__ void k_bin_scatter(const double* __restrict__ lam, int64_t M, double 
     }
 }
 
-// colptr[t * ncb + k] = start of column bin k of tile t (= scan at its first row key).
-__global__ void k_colptr(const int* __restrict__ offs, int64_t nbins, int ncb, int total,
-                         int* __restrict__ colptr) {
+// What the host needs of a binning: sum[0] entries, [1] the status word, [2] block chunks (0 when
+// there are none), [3] unused, then the entries of each tile, then one byte per grid column: some
+// run of taps starts there. Before the scatter: colptr[t * ncb + k] = start of column bin k of tile
+// t (= scan at its first row key), colptr[nbins] = entries.
+constexpr int kSumHead = 4;
+__global__ void k_bin_summary(const int* __restrict__ offs, const int* __restrict__ hist,
+                              int64_t nbins, int ncb, int G, int T, int W, int ntx,
+                              const unsigned* __restrict__ status, int* __restrict__ colptr,
+                              int* __restrict__ sum, unsigned char* __restrict__ first) {
+    const int total = offs[nbins * ncb - 1] + hist[nbins * ncb - 1];
+    auto start = [&](int64_t bin) { return bin < nbins ? offs[bin * ncb] : total; };
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= nbins;
-         i += (int64_t)gridDim.x * blockDim.x)
-        colptr[i] = i < nbins ? offs[i * ncb] : total;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int at = start(i);
+        colptr[i] = at;
+        if (i == nbins) {
+            sum[0] = total;
+            sum[1] = (int)*status;
+            continue;
+        }
+        const int64_t tile = i / ncb;
+        const int k = (int)(i - tile * ncb);
+        if (k == 0) sum[kSumHead + tile] = start(i + ncb) - at;
+        if (start(i + 1) > at) {
+            int x = (int)(tile % ntx) * T + k - (W - 1);
+            if (x < 0) x += G;
+            if (x >= G) x -= G;
+            first[x] = 1;
+        }
+    }
 }
 
 // ---- exclusive scan of int32 (three phases: block sums, scan of sums, block rescan) ----------
@@ -198,12 +231,31 @@ __device__ __forceinline__ int block_exclusive_sum(int v, int* total) {
     return before;
 }
 
+// a thread's consecutive items, 16 bytes at a time (the arrays are allocations: aligned)
+__device__ __forceinline__ void scan_load(const int* __restrict__ in, int64_t base, int64_t n,
+                                          int (&v)[kScanItems]) {
+    if (base + kScanItems <= n) {
+#pragma unroll
+        for (int i = 0; i < kScanItems; i += 4) {
+            const int4 q = *reinterpret_cast<const int4*>(in + base + i);
+            v[i] = q.x;
+            v[i + 1] = q.y;
+            v[i + 2] = q.z;
+            v[i + 3] = q.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i) v[i] = base + i < n ? in[base + i] : 0;
+    }
+}
+
 __global__ void k_scan_sums(const int* __restrict__ in, int64_t n, int* __restrict__ bsum) {
     int64_t base = (int64_t)blockIdx.x * kScanBlock + (int64_t)threadIdx.x * kScanItems;
+    int vals[kScanItems];
+    scan_load(in, base, n, vals);
     int s = 0;
 #pragma unroll
-    for (int i = 0; i < kScanItems; ++i)
-        if (base + i < n) s += in[base + i];
+    for (int i = 0; i < kScanItems; ++i) s += vals[i];
     int total;
     block_exclusive_sum(s, &total);
     if (threadIdx.x == 0) bsum[blockIdx.x] = total;
@@ -236,18 +288,27 @@ __global__ void k_scan_apply(const int* __restrict__ in, int64_t n, const int* _
                              int* __restrict__ out) {
     int64_t base = (int64_t)blockIdx.x * kScanBlock + (int64_t)threadIdx.x * kScanItems;
     int vals[kScanItems];
+    scan_load(in, base, n, vals);
     int s = 0;
 #pragma unroll
-    for (int i = 0; i < kScanItems; ++i) {
-        vals[i] = (base + i < n) ? in[base + i] : 0;
-        s += vals[i];
-    }
+    for (int i = 0; i < kScanItems; ++i) s += vals[i];
     int total;
     int run = block_exclusive_sum(s, &total) + boff[blockIdx.x];
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i) {
-        if (base + i < n) out[base + i] = run;
-        run += vals[i];
+        const int v = vals[i];
+        vals[i] = run;
+        run += v;
+    }
+    if (base + kScanItems <= n) {
+#pragma unroll
+        for (int i = 0; i < kScanItems; i += 4)
+            *reinterpret_cast<int4*>(out + base + i) =
+                make_int4(vals[i], vals[i + 1], vals[i + 2], vals[i + 3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i)
+            if (base + i < n) out[base + i] = vals[i];
     }
 }
 
@@ -275,11 +336,11 @@ ftcg_status_t exclusive_scan_i32(const int* d_in, int* d_out, int64_t n, cudaStr
 
 void free_binning(Binning& b) {
     free_chunks(b);
-    if (b.ent) cudaFree(b.ent);
-    if (b.colptr) cudaFree(b.colptr);
-    if (b.tile_order) cudaFree(b.tile_order);
-    if (b.halo_buf) cudaFree(b.halo_buf);
-    if (b.tile_full) cudaFree(b.tile_full);
+    pool_free(b.ent, nullptr);
+    pool_free(b.colptr, nullptr);
+    pool_free(b.tile_order, nullptr);
+    pool_free(b.halo_buf, nullptr);
+    pool_free(b.tile_full, nullptr);
     b.halo_buf = nullptr;
     b.tile_full = nullptr;
     b.ent = nullptr;
@@ -291,38 +352,28 @@ void free_binning(Binning& b) {
 
 // Launch order of the tiles: decreasing entry count, so that the heaviest tiles start first and
 // the light (often empty) ones fill the tail.
-static ftcg_status_t order_tiles(Binning& b, cudaStream_t s, int64_t* bytes) {
-    const int64_t nbins = (int64_t)b.ntiles * b.ncb;
-    std::vector<int> cp(nbins + 1);
-    FTCG_CK(cudaMemcpyAsync(cp.data(), b.colptr, (nbins + 1) * sizeof(int), cudaMemcpyDeviceToHost,
-                            s));
-    FTCG_CK(cudaStreamSynchronize(s));
-    b.tile_cnt.resize(b.ntiles);
-    for (int t = 0; t < b.ntiles; ++t)
-        b.tile_cnt[t] = cp[(int64_t)(t + 1) * b.ncb] - cp[(int64_t)t * b.ncb];
+// tile_cnt is set; first[x]: some run of taps starts in grid column x.
+static ftcg_status_t order_tiles(Binning& b, const unsigned char* first, cudaStream_t s,
+                                 int64_t* bytes) {
+    // stable counting sort by decreasing count, 11 bits at a time
     std::vector<int>& order = b.h_order;
     order.resize(b.ntiles);
     std::iota(order.begin(), order.end(), 0);
     auto cnt = [&](int t) { return b.tile_cnt[t]; };
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cnt(x) > cnt(y); });
+    const int top = *std::max_element(b.tile_cnt.begin(), b.tile_cnt.end());
+    std::vector<int> tmp(b.ntiles), at(2049);
+    for (int shift = 0; (top >> shift) > 0; shift += 11) {
+        auto digit = [&](int t) { return 2047 - ((cnt(t) >> shift) & 2047); };
+        std::fill(at.begin(), at.end(), 0);
+        for (int t : order) ++at[digit(t) + 1];
+        for (int k = 0; k < 2048; ++k) at[k + 1] += at[k];
+        for (int t : order) tmp[at[digit(t)]++] = t;
+        order.swap(tmp);
+    }
     b.n_nonempty = 0;
     while (b.n_nonempty < b.ntiles && cnt(order[b.n_nonempty]) > 0) ++b.n_nonempty;
-    // grid columns that taps reach: an entry in column bin k of tile column tx has its first tap
-    // (of the tile's run) at X0 + k - (w - 1), and the sample's taps of that run follow it
-    std::vector<unsigned char> first(b.G, 0);   // columns where some run of taps starts
-    for (int i = 0; i < b.n_nonempty; ++i) {
-        const int t = order[i];
-        const int X0 = (t % b.ntx) * b.T;
-        const int64_t base = (int64_t)t * b.ncb;
-        for (int k = 0; k < b.ncb; ++k) {
-            if (cp[base + k + 1] == cp[base + k]) continue;
-            int x = X0 + k - (b.W - 1);
-            if (x < 0) x += b.G;
-            if (x >= b.G) x -= b.G;
-            first[x] = 1;
-        }
-    }
-    b.col_occ.assign(b.G, 0);                    // the w columns from each start (mod G)
+    // grid columns that taps reach: the w columns from each start (mod G)
+    b.col_occ.assign(b.G, 0);
     for (int x = 0, run = 0; x < b.G + b.W - 1; ++x) {
         run = first[x % b.G] ? b.W : run - 1;
         if (run > 0) b.col_occ[x % b.G] = 1;
@@ -357,8 +408,8 @@ static ftcg_status_t order_tiles(Binning& b, cudaStream_t s, int64_t* bytes) {
 }
 
 ftcg_status_t build_binning(Binning& b, const double* d_lambda, int64_t M, double scale, int G,
-                            int T, int W, bool halo, unsigned* d_status, int4* d_samp,
-                            cudaStream_t s, int64_t* bytes) {
+                            int T, int W, bool halo, bool block_chunks, unsigned* d_status,
+                            int4* d_samp, cudaStream_t s, int64_t* bytes, unsigned* status) {
     b.G = G;
     b.T = T;
     b.W = W;
@@ -366,6 +417,7 @@ ftcg_status_t build_binning(Binning& b, const double* d_lambda, int64_t M, doubl
     b.ntx = (G + T - 1) / T;
     b.ntiles = b.ntx * b.ntx;
     b.ncb = T + W - 1;
+    *status = 0;
     const int64_t nbins = (int64_t)b.ntiles * b.ncb;      // (tile, column bin)
     const int64_t nkeys = nbins * b.ncb;                  // (tile, column bin, row)
     FTCG_CK(pool_malloc(&b.colptr, (nbins + 1) * sizeof(int), s));
@@ -373,39 +425,65 @@ ftcg_status_t build_binning(Binning& b, const double* d_lambda, int64_t M, doubl
     if (M == 0) {
         FTCG_CK(cudaMemsetAsync(b.colptr, 0, (nbins + 1) * sizeof(int), s));
         b.n_entries = 0;
-        return FTCG_SUCCESS;
+        return block_chunks ? finish_block_chunks(b, nullptr, nullptr, nullptr, 0, s, bytes)
+                            : FTCG_SUCCESS;
     }
+    // device temporaries in one allocation: key counts and offsets, the block chunks' counts and
+    // offsets, the summary
+    const int64_t nseg = block_chunks ? (int64_t)b.ntiles * (T / 8) * (T / 8) : 0;
+    const size_t sum_ints = kSumHead + (size_t)b.ntiles + (size_t)(G + 3) / 4;
+    auto up4 = [](int64_t n) { return (n + 3) / 4 * 4; };      // keep 16-byte alignment
     int* hist = nullptr;
-    int* offs = nullptr;
-    FTCG_CK(pool_malloc(&hist, nkeys * sizeof(int), s));
-    FTCG_CK(pool_malloc(&offs, nkeys * sizeof(int), s));
-    FTCG_CK(cudaMemsetAsync(hist, 0, nkeys * sizeof(int), s));
-    k_bin_count<<<grid_for(M), kThreads, 0, s>>>(d_lambda, M, scale, G, T, W, b.ntx, b.ncb, halo,
-                                                 hist, d_status, d_samp);
-    FTCG_CK(cudaGetLastError());
-    FTCG_TRY(exclusive_scan_i32(hist, offs, nkeys, s));
-    int last_off = 0, last_cnt = 0;
-    FTCG_CK(cudaMemcpyAsync(&last_off, offs + nkeys - 1, sizeof(int), cudaMemcpyDeviceToHost, s));
-    FTCG_CK(cudaMemcpyAsync(&last_cnt, hist + nkeys - 1, sizeof(int), cudaMemcpyDeviceToHost, s));
-    FTCG_CK(cudaStreamSynchronize(s));
-    const int total = last_off + last_cnt;
-    b.n_entries = total;
-    k_colptr<<<grid_for(nbins + 1), kThreads, 0, s>>>(offs, nbins, b.ncb, total, b.colptr);
-    FTCG_CK(cudaGetLastError());
-    if (total > 0) {
-        FTCG_CK(pool_malloc(&b.ent, (size_t)(total + kEntryPad) * sizeof(Entry), s));
-        *bytes += (int64_t)(total + kEntryPad) * sizeof(Entry);
-        FTCG_CK(cudaMemsetAsync(b.ent + total, 0, kEntryPad * sizeof(Entry), s));
-        k_bin_scatter<<<grid_for(M), kThreads, 0, s>>>(d_lambda, M, scale, G, T, W, b.ntx, b.ncb,
-                                                       halo, offs, b.ent);
+    FTCG_CK(pool_malloc(&hist, (2 * up4(nkeys) + 2 * up4(nseg) + sum_ints) * sizeof(int), s));
+    int* offs = hist + up4(nkeys);
+    int* seg_cnt = offs + up4(nkeys);
+    int* seg_off = seg_cnt + up4(nseg);
+    int* sum = seg_off + up4(nseg);
+    unsigned char* first = reinterpret_cast<unsigned char*>(sum + kSumHead + b.ntiles);
+    auto run = [&]() -> ftcg_status_t {
+        FTCG_CK(cudaMemsetAsync(hist, 0, nkeys * sizeof(int), s));
+        FTCG_CK(cudaMemsetAsync(sum, 0, sum_ints * sizeof(int), s));
+        k_bin_count<<<grid_for(M), kThreads, 0, s>>>(d_lambda, M, scale, G, T, W, b.ntx, b.ncb,
+                                                     halo, hist, d_status, d_samp);
+        FTCG_CK(cudaGetLastError());
+        FTCG_TRY(exclusive_scan_i32(hist, offs, nkeys, s));
+        k_bin_summary<<<grid_for(nbins + 1), kThreads, 0, s>>>(offs, hist, nbins, b.ncb, G, T, W,
+                                                               b.ntx, d_status, b.colptr, sum,
+                                                               first);
+        FTCG_CK(cudaGetLastError());
+        if (block_chunks)
+            FTCG_TRY(count_block_chunks(b, offs, nkeys, sum, seg_cnt, seg_off, sum + 2, s));
+        int64_t room = M;                                 // halo layout: at most one per sample
+        if (!halo) {
+            int total = 0;
+            FTCG_CK(cudaMemcpyAsync(&total, sum, sizeof(int), cudaMemcpyDeviceToHost, s));
+            FTCG_CK(cudaStreamSynchronize(s));
+            room = total;
+        }
+        FTCG_CK(pool_malloc(&b.ent, (size_t)(room + kEntryPad) * sizeof(Entry), s));
+        *bytes += (int64_t)(room + kEntryPad) * sizeof(Entry);
+        k_bin_scatter<<<grid_for(M), kThreads, 0, s>>>(d_samp, M, G, T, W, b.ntx, b.ncb, halo, offs,
+                                                       sum, b.ent);
         FTCG_CK(cudaGetLastError());
         if (b.det) {
             k_key_sort<<<grid_for(nkeys), kThreads, 0, s>>>(hist, offs, nkeys, b.ent);
             FTCG_CK(cudaGetLastError());
         }
-    }
-    FTCG_CK(pool_free(hist, s));
-    FTCG_CK(pool_free(offs, s));
+        std::vector<int> h(sum_ints);
+        FTCG_CK(cudaMemcpyAsync(h.data(), sum, sum_ints * sizeof(int), cudaMemcpyDeviceToHost, s));
+        FTCG_CK(cudaStreamSynchronize(s));
+        b.n_entries = h[0];
+        *status = (unsigned)h[1];
+        b.tile_cnt.assign(h.begin() + kSumHead, h.begin() + kSumHead + b.ntiles);
+        FTCG_TRY(order_tiles(b, reinterpret_cast<unsigned char*>(h.data() + kSumHead + b.ntiles), s,
+                             bytes));
+        if (block_chunks)
+            FTCG_TRY(finish_block_chunks(b, offs, seg_cnt, seg_off, h[2], s, bytes));
+        return FTCG_SUCCESS;
+    };
+    const ftcg_status_t st = run();
+    pool_free(hist, s);
+    FTCG_TRY(st);
     if (halo) {
         // per tile: the right strip (T + w - 1) x (w - 1) and the bottom strip (w - 1) x T
         b.halo_cells = (T + W - 1) * (W - 1) + (W - 1) * T;
@@ -413,7 +491,7 @@ ftcg_status_t build_binning(Binning& b, const double* d_lambda, int64_t M, doubl
         FTCG_CK(pool_malloc(&b.halo_buf, hb, s));
         *bytes += (int64_t)hb;
     }
-    return order_tiles(b, s, bytes);
+    return FTCG_SUCCESS;
 }
 
 }  // namespace ftcg

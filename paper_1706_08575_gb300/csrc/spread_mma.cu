@@ -36,6 +36,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 
 #include "spread_blk.cuh"
 #include "spread_mma.cuh"
@@ -48,10 +49,51 @@ constexpr double kMmaPolyBound = 1e-6;
 
 }  // namespace
 
+namespace {
+bool fit_window_poly(int W, double beta, int kind, MmaPoly* out, double* max_err);
+
+// The last fits (a ring of 16), by window: a fit evaluates the FP64 window about 2000 times on the
+// host (50 us), and a stream of pings asks for the same one with every plan.
+struct PolyFit {
+    int W = -1, kind = 0;
+    double beta = 0, err = 0;
+    bool ok = false;
+    MmaPoly poly;
+};
+std::mutex g_fit_mu;
+PolyFit g_fit[16];
+int g_fit_next = 0;
+}  // namespace
+
+bool mma_window_poly(int W, double beta, int kind, MmaPoly* out, double* max_err) {
+    {
+        std::lock_guard<std::mutex> lk(g_fit_mu);
+        for (const PolyFit& f : g_fit)
+            if (f.W == W && f.kind == kind && f.beta == beta) {
+                *out = f.poly;
+                *max_err = f.err;
+                return f.ok;
+            }
+    }
+    PolyFit f;
+    f.ok = fit_window_poly(W, beta, kind, &f.poly, &f.err);
+    f.W = W;
+    f.kind = kind;
+    f.beta = beta;
+    *out = f.poly;
+    *max_err = f.err;
+    std::lock_guard<std::mutex> lk(g_fit_mu);
+    g_fit[g_fit_next] = f;
+    g_fit_next = (g_fit_next + 1) % 16;
+    return f.ok;
+}
+
+namespace {
+
 // Chebyshev interpolation of phi(s + w/2 - 1/2 - l) on s in [-1/2, 1/2] at the 8 Chebyshev
 // points (phi the plan's window, in FP64), converted to monomial coefficients in s. The error is
 // measured on 257 points per tap.
-bool mma_window_poly(int W, double beta, int kind, MmaPoly* out, double* max_err) {
+bool fit_window_poly(int W, double beta, int kind, MmaPoly* out, double* max_err) {
     std::memset(out, 0, sizeof(*out));
     *max_err = 0.0;
     if (W > kMmaMaxW || W < 2) {
@@ -108,8 +150,6 @@ bool mma_window_poly(int W, double beta, int kind, MmaPoly* out, double* max_err
     *max_err = worst;
     return worst <= kMmaPolyBound;
 }
-
-namespace {
 
 // ---- chunk construction (plan time) ----------------------------------------------------------
 // The greedy walk over one (tile, column bin) segment, entries sorted by first-tap row r:
@@ -253,61 +293,89 @@ ftcg_status_t dispatch_mma_t(const Plan& p, const void* vals, float2* grid, cuda
     return run_mma<64, VBF, ABF>(p, vals, grid, s, nt);
 }
 
-// ---- block chunks (plan time): one thread per (tile, 8 x 8 block of first-tap cells) ----------
-// The block's entries are those of its 8 column bins (halo layout: bin = first-tap column + w - 1)
-// whose first-tap row lies in the block's 8 rows, taken bin by bin in row order (deterministic).
-__device__ __forceinline__ int blk_row(const Entry& e, int W) {
-    return (int)(e.packed >> kSampleBits) - (W - 1);
+// ---- block chunks (plan time) --------------------------------------------------------------
+// The entries of block (bx, by) of a tile are, in each of its 8 column bins (halo layout: bin =
+// first-tap column + w - 1), the contiguous keys of its 8 first-tap rows, so counts and places come
+// from the sort's key offsets; bins follow one another in order (deterministic). Large ping, us:
+// reading every entry once per block row to count and again to emit 80 + 149 (T = 32) or 145 + 278
+// (T = 64), here 6 + 18.
+// keys of rows 8 by .. 8 by + 7 of bin 8 bx + b of tile: the first key and one past the last
+__device__ __forceinline__ int64_t blk_key(int64_t tile, int ncb, int bx, int by, int b, int W) {
+    return (tile * ncb + 8 * bx + b + W - 1) * ncb + 8 * by + W - 1;
 }
 
-__global__ void k_blk_count(const Entry* __restrict__ ent, const int* __restrict__ colptr,
-                            int ntiles, int ncb, int T, int W, int* __restrict__ cnt) {
+// Chunks per (tile, block) from the key starts (before the scatter); total: the entries.
+__global__ void k_blk_count(const int* __restrict__ start, int64_t nkeys,
+                            const int* __restrict__ total, int ntiles, int ncb, int T, int W,
+                            int* __restrict__ cnt) {
     const int nbs = T / 8, nb = nbs * nbs;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (int64_t)ntiles * nb;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t tile = i / nb;
-        const int b = (int)(i - tile * nb), bxi = b % nbs, byi = b / nbs;
+        const int b = (int)(i - tile * nb), bx = b % nbs, by = b / nbs;
         int c = 0;
-        for (int bin = 8 * bxi + W - 1; bin < 8 * bxi + 8 + W - 1 && bin < ncb; ++bin) {
-            const int a0 = colptr[tile * ncb + bin], a1 = colptr[tile * ncb + bin + 1];
-            for (int e = a0; e < a1; ++e) c += (blk_row(ent[e], W) >> 3) == byi;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int64_t key = blk_key(tile, ncb, bx, by, k, W);
+            c += (key + 8 < nkeys ? start[key + 8] : *total) - start[key];
         }
         cnt[i] = (c + kMmaChunk - 1) / kMmaChunk;
     }
 }
 
-__global__ void k_blk_emit(const Entry* __restrict__ ent, const int* __restrict__ colptr,
-                           const int* __restrict__ off, int ntiles, int ncb, int T, int W,
-                           MmaEntry* __restrict__ cent, uint32_t* __restrict__ chdr) {
-    const int nbs = T / 8, nb = nbs * nbs;
+// *out = chunks in all
+__global__ void k_blk_total(const int* __restrict__ cnt, const int* __restrict__ off, int64_t nseg,
+                            int* __restrict__ out) {
+    *out = off[nseg - 1] + cnt[nseg - 1];
+}
+
+// One warp per (tile, block); end: the key ends (after the scatter), so key k starts at end[k - 1].
+__global__ void __launch_bounds__(256)
+    k_blk_emit(const Entry* __restrict__ ent, const int* __restrict__ end,
+               const int* __restrict__ cnt, const int* __restrict__ off, int ntiles, int ncb, int T,
+               int W, MmaEntry* __restrict__ cent, uint32_t* __restrict__ chdr) {
+    const int nbs = T / 8, nb = nbs * nbs, lane = threadIdx.x & 31;
     const float c0 = 0.5f * W - 0.5f;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (int64_t)ntiles * nb;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t tile = i / nb;
-        const int b = (int)(i - tile * nb), bxi = b % nbs, byi = b / nbs;
-        const int64_t first = off[i];
-        int64_t k = 0;
-        for (int bin = 8 * bxi + W - 1; bin < 8 * bxi + 8 + W - 1 && bin < ncb; ++bin) {
-            const int a0 = colptr[tile * ncb + bin], a1 = colptr[tile * ncb + bin + 1];
-            const int ox = bin - (W - 1) - 8 * bxi;              // first-tap column in the block
-            for (int e = a0; e < a1; ++e) {
-                const Entry en = ent[e];
-                const int r = blk_row(en, W);
-                if ((r >> 3) != byi) continue;
-                MmaEntry m;
-                m.sx = en.dx - c0;                              // as the column chunks
+    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+         i < (int64_t)ntiles * nb; i += nw) {
+        const int nch = cnt[i];
+        if (nch == 0) continue;
+        const int64_t tile = i / nb, first = off[i];
+        const int b = (int)(i - tile * nb), bx = b % nbs, by = b / nbs;
+        int s0 = 0, n = 0;
+        if (lane < 8) {                                // lane k: bin k's entries
+            const int64_t key = blk_key(tile, ncb, bx, by, lane, W);
+            s0 = key > 0 ? end[key - 1] : 0;
+            n = end[key + 7] - s0;
+        }
+        int upto = n;                                  // inclusive prefix over the bins
+        for (int o = 1; o < 8; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, upto, o);
+            if (lane >= o) upto += v;
+        }
+        const int total = __shfl_sync(0xffffffffu, upto, 7);
+        for (int e0 = 0; e0 < nch * kMmaChunk; e0 += 32) {
+            const int e = e0 + lane;
+            int bin = 0;
+#pragma unroll
+            for (int k = 0; k < 7; ++k) bin += e >= __shfl_sync(0xffffffffu, upto, k);
+            const int src = __shfl_sync(0xffffffffu, s0 - (upto - n), bin) + e;
+            if (e >= nch * kMmaChunk) continue;
+            MmaEntry m{0.f, 0.f, 0u, kMmaPad};
+            if (e < total) {
+                const Entry en = ent[src];
+                const int r = (int)(en.packed >> kSampleBits) - (W - 1);
+                m.sx = en.dx - c0;                     // as the column chunks
                 m.sy = en.dy - c0;
                 m.alpha = en.alpha;
-                m.packed = (en.packed & kSampleMask) | ((uint32_t)ox << blk::kOffXShift) |
-                           ((uint32_t)(r - 8 * byi) << blk::kOffYShift);
-                cent[first * kMmaChunk + k] = m;
-                ++k;
+                m.packed = (en.packed & kSampleMask) | ((uint32_t)bin << blk::kOffXShift) |
+                           ((uint32_t)(r - 8 * by) << blk::kOffYShift);
             }
+            cent[first * kMmaChunk + e] = m;
         }
-        const int64_t nch = (k + kMmaChunk - 1) / kMmaChunk;
-        for (; k < nch * kMmaChunk; ++k) cent[first * kMmaChunk + k] = MmaEntry{0.f, 0.f, 0u, kMmaPad};
-        for (int64_t c = 0; c < nch; ++c)
-            chdr[first + c] = (uint32_t)(8 * bxi) | ((uint32_t)(8 * byi) << 8);
+        for (int c = lane; c < nch; c += 32)
+            chdr[first + c] = (uint32_t)(8 * bx) | ((uint32_t)(8 * by) << 8);
     }
 }
 
@@ -348,9 +416,9 @@ ftcg_status_t dispatch_blk_t(const Plan& p, const void* vals, float2* grid, cuda
 }  // namespace
 
 void free_chunks(Binning& b) {
-    if (b.cent) cudaFree(b.cent);
-    if (b.chdr) cudaFree(b.chdr);
-    if (b.tile_chunk) cudaFree(b.tile_chunk);
+    pool_free(b.cent, nullptr);
+    pool_free(b.chdr, nullptr);
+    pool_free(b.tile_chunk, nullptr);
     b.cent = nullptr;
     b.chdr = nullptr;
     b.tile_chunk = nullptr;
@@ -359,15 +427,62 @@ void free_chunks(Binning& b) {
     b.blk = false;
 }
 
-ftcg_status_t build_chunks(Binning& b, cudaStream_t s, int64_t* bytes, bool block) {
-    if (!b.halo || b.W > kMmaMaxW || (b.T != 32 && b.T != 64)) {
-        set_error("build_chunks: the tensor-core path needs the halo layout, w <= 8, T = 32 or 64");
-        return FTCG_ERR_NOT_SUPPORTED;
-    }
-    b.blk = block;
-    // segments: (tile, column bin) for column chunks, (tile, 8 x 8 block) for block chunks
-    const int per_tile = block ? (b.T / 8) * (b.T / 8) : b.ncb;
+namespace {
+
+// room for total chunks and the padding ones after them (slots flagged as padding)
+ftcg_status_t alloc_chunks(Binning& b, int total, cudaStream_t s, int64_t* bytes) {
+    b.n_chunks = total;
+    constexpr int kPad = mma::kPrefetchChunks;
+    const size_t ent_bytes = (size_t)(total + kPad) * kMmaChunk * sizeof(MmaEntry);
+    FTCG_CK(pool_malloc(&b.cent, ent_bytes, s));
+    FTCG_CK(pool_malloc(&b.chdr, (size_t)(total + kPad) * sizeof(uint32_t), s));
+    *bytes += (int64_t)ent_bytes + (int64_t)(total + kPad) * sizeof(uint32_t);
+    k_pad_chunks<<<1, kPad * kMmaChunk, 0, s>>>(b.cent + (size_t)total * kMmaChunk,
+                                                kPad * kMmaChunk);
+    FTCG_CK(cudaGetLastError());
+    FTCG_CK(cudaMemsetAsync(b.chdr + total, 0, kPad * sizeof(uint32_t), s));
+    return FTCG_SUCCESS;
+}
+
+}  // namespace
+
+ftcg_status_t count_block_chunks(const Binning& b, const int* start, int64_t nkeys,
+                                 const int* d_entries, int* cnt, int* off, int* d_total,
+                                 cudaStream_t s) {
+    const int64_t nseg = (int64_t)b.ntiles * (b.T / 8) * (b.T / 8);
+    k_blk_count<<<blocks_for(nseg, 256), 256, 0, s>>>(start, nkeys, d_entries, b.ntiles, b.ncb, b.T,
+                                                      b.W, cnt);
+    FTCG_CK(cudaGetLastError());
+    FTCG_TRY(exclusive_scan_i32(cnt, off, nseg, s));
+    k_blk_total<<<1, 1, 0, s>>>(cnt, off, nseg, d_total);
+    FTCG_CK(cudaGetLastError());
+    return FTCG_SUCCESS;
+}
+
+ftcg_status_t finish_block_chunks(Binning& b, const int* end, const int* cnt, const int* off,
+                                  int total, cudaStream_t s, int64_t* bytes) {
+    const int per_tile = (b.T / 8) * (b.T / 8);
     const int64_t nseg = (int64_t)b.ntiles * per_tile;
+    b.blk = b.mma = true;
+    FTCG_CK(pool_malloc(&b.tile_chunk, (b.ntiles + 1) * sizeof(int), s));
+    *bytes += (b.ntiles + 1) * sizeof(int);
+    if (b.n_entries == 0) {
+        FTCG_CK(cudaMemsetAsync(b.tile_chunk, 0, (b.ntiles + 1) * sizeof(int), s));
+        b.n_chunks = 0;
+        return FTCG_SUCCESS;
+    }
+    FTCG_TRY(alloc_chunks(b, total, s, bytes));
+    k_blk_emit<<<blocks_for(nseg, 8), 256, 0, s>>>(b.ent, end, cnt, off, b.ntiles, b.ncb, b.T, b.W,
+                                                   b.cent, b.chdr);
+    FTCG_CK(cudaGetLastError());
+    k_tile_chunk<<<blocks_for(b.ntiles + 1, 256), 256, 0, s>>>(off, b.ntiles, per_tile, total,
+                                                               b.tile_chunk);
+    FTCG_CK(cudaGetLastError());
+    return FTCG_SUCCESS;
+}
+
+ftcg_status_t build_column_chunks(Binning& b, cudaStream_t s, int64_t* bytes) {
+    const int64_t nseg = (int64_t)b.ntiles * b.ncb;    // (tile, column bin)
     FTCG_CK(pool_malloc(&b.tile_chunk, (b.ntiles + 1) * sizeof(int), s));
     *bytes += (b.ntiles + 1) * sizeof(int);
     if (b.n_entries == 0) {
@@ -380,11 +495,7 @@ ftcg_status_t build_chunks(Binning& b, cudaStream_t s, int64_t* bytes, bool bloc
     int* off = nullptr;
     FTCG_CK(pool_malloc(&cnt, nseg * sizeof(int), s));
     FTCG_CK(pool_malloc(&off, nseg * sizeof(int), s));
-    if (block)
-        k_blk_count<<<blocks_for(nseg, 256), 256, 0, s>>>(b.ent, b.colptr, b.ntiles, b.ncb, b.T,
-                                                          b.W, cnt);
-    else
-        k_chunk_count<<<blocks_for(nseg, 256), 256, 0, s>>>(b.ent, b.colptr, nseg, b.W, cnt);
+    k_chunk_count<<<blocks_for(nseg, 256), 256, 0, s>>>(b.ent, b.colptr, nseg, b.W, cnt);
     FTCG_CK(cudaGetLastError());
     FTCG_TRY(exclusive_scan_i32(cnt, off, nseg, s));
     int last_off = 0, last_cnt = 0;
@@ -392,25 +503,11 @@ ftcg_status_t build_chunks(Binning& b, cudaStream_t s, int64_t* bytes, bool bloc
     FTCG_CK(cudaMemcpyAsync(&last_cnt, cnt + nseg - 1, sizeof(int), cudaMemcpyDeviceToHost, s));
     FTCG_CK(cudaStreamSynchronize(s));
     const int total = last_off + last_cnt;
-    b.n_chunks = total;
-    // padding chunks after the last (slots flagged as padding), for the kernel's reads ahead
-    constexpr int kPad = mma::kPrefetchChunks;
-    const size_t ent_bytes = (size_t)(total + kPad) * kMmaChunk * sizeof(MmaEntry);
-    FTCG_CK(pool_malloc(&b.cent, ent_bytes, s));
-    FTCG_CK(pool_malloc(&b.chdr, (size_t)(total + kPad) * sizeof(uint32_t), s));
-    *bytes += (int64_t)ent_bytes + (int64_t)(total + kPad) * sizeof(uint32_t);
-    k_pad_chunks<<<1, kPad * kMmaChunk, 0, s>>>(b.cent + (size_t)total * kMmaChunk,
-                                                kPad * kMmaChunk);
+    FTCG_TRY(alloc_chunks(b, total, s, bytes));
+    k_chunk_emit<<<blocks_for(nseg, 256), 256, 0, s>>>(b.ent, b.colptr, off, nseg, b.ncb, b.W,
+                                                       b.cent, b.chdr);
     FTCG_CK(cudaGetLastError());
-    FTCG_CK(cudaMemsetAsync(b.chdr + total, 0, kPad * sizeof(uint32_t), s));
-    if (block)
-        k_blk_emit<<<blocks_for(nseg, 256), 256, 0, s>>>(b.ent, b.colptr, off, b.ntiles, b.ncb,
-                                                         b.T, b.W, b.cent, b.chdr);
-    else
-        k_chunk_emit<<<blocks_for(nseg, 256), 256, 0, s>>>(b.ent, b.colptr, off, nseg, b.ncb, b.W,
-                                                           b.cent, b.chdr);
-    FTCG_CK(cudaGetLastError());
-    k_tile_chunk<<<blocks_for(b.ntiles + 1, 256), 256, 0, s>>>(off, b.ntiles, per_tile, total,
+    k_tile_chunk<<<blocks_for(b.ntiles + 1, 256), 256, 0, s>>>(off, b.ntiles, b.ncb, total,
                                                                b.tile_chunk);
     FTCG_CK(cudaGetLastError());
     FTCG_CK(pool_free(cnt, s));
