@@ -87,6 +87,26 @@ __device__ __forceinline__ void stage_block_slot(const MmaEntry& e, float2 v, bo
     q = (((e.packed >> kOffXShift) & 7u) << 2) | (((e.packed >> kOffYShift) & 7u) << 18);
 }
 
+// *cell(k) += v[k], k = 0..7, atomically, in shared memory. An FP32 shared atomicAdd is a loop of load,
+// add and compare-and-swap on this GPU, and eight of them wait for one another; here the eight
+// loads and then the eight swaps are in flight together, and only a cell that another warp
+// changed in between (rare) takes the loop. With the bank order of the flush below: 64-ping batch
+// (a flush every other chunk) spreading 980 -> 895 us, BF16 precision raster 152 -> 146; the dense ping
+// unchanged (71 us).
+template <typename Cell>
+__device__ __forceinline__ void shared_add8(const Cell& cell, const float (&v)[8]) {
+    unsigned seen[8], got[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) seen[k] = *reinterpret_cast<volatile unsigned*>(cell(k));
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        got[k] = atomicCAS(reinterpret_cast<unsigned*>(cell(k)), seen[k],
+                           __float_as_uint(__uint_as_float(seen[k]) + v[k]));
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        if (got[k] != seen[k]) atomicAdd(cell(k), v[k]);
+}
+
 // One halo-layout tile by the whole CTA (kThreads threads): its block chunks
 // [tile_chunk[tile], tile_chunk[tile + 1]) split into contiguous ranges, one per warp (or all to
 // warp 0 with one_warp); then the tile and its overflow strips are stored. smem: blk::tile_smem_bytes(T).
@@ -135,14 +155,28 @@ __device__ __forceinline__ void spread_tile(const MmaEntry* __restrict__ cent,
     uint32_t cur = 0xffffffffu;                // the block in the fragments (its header)
     // one plane's window quadrants from its partial sums, added to the accumulator at o
     auto flush_plane = [&](float* acc, int o, float (&d0)[4], float (&d1)[4]) {
+        float v[8];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            const float q10 = d0[2 + j] - d0[j];
-            atomicAdd(acc + o + j, d0[j]);
-            atomicAdd(acc + o + 8 * LD + j, q10);
-            atomicAdd(acc + o + 8 + j, d1[j] - d0[j]);
-            atomicAdd(acc + o + 8 * LD + 8 + j, (d1[2 + j] - d1[j]) - q10);
+            v[j] = d0[j];
+            v[2 + j] = d0[2 + j] - d0[j];
+            v[4 + j] = d1[j] - d0[j];
+            v[6 + j] = (d1[2 + j] - d1[j]) - v[2 + j];
         }
+        // rows g >= 4 take their two columns in the other order: LD is 8 mod 32, so that their
+        // cells' banks are then the odd ones while rows g < 4 use the even ones
+        const int sw = g >> 2;
+#pragma unroll
+        for (int k = 0; k < 8; k += 2) {
+            const float a = sw ? v[k + 1] : v[k], b = sw ? v[k] : v[k + 1];
+            v[k] = a;
+            v[k + 1] = b;
+        }
+        auto cell = [&](int k) {
+            return acc + o + ((k & 1) ? 1 - sw : sw) + ((k & 2) ? 8 * LD : 0) + ((k & 4) ? 8 : 0);
+        };
+        static_assert(LD % 32 == 8, "bank order of the flush");
+        shared_add8(cell, v);
 #pragma unroll
         for (int q = 0; q < 4; ++q) d0[q] = d1[q] = 0.f;
     };
