@@ -288,7 +288,7 @@ struct Batch {
         float2* grids = nullptr;
         cufftHandle fft = 0;
         bool fft_ok = false;
-        // shared-memory FFT (power-of-two G in 256..4096): twiddle tables, (ping, column block)
+        // shared-memory FFT (power-of-two G in 64..4096): twiddle tables, (ping, column block)
         // items of the column pass, and the class's pings for the row pass
         bool smem = false;
         float2* tw = nullptr;
@@ -401,6 +401,8 @@ ftcg_status_t launch_class_fft_t(Batch& b, const Batch::Class& c, cudaStream_t s
 
 ftcg_status_t launch_class_fft(Batch& b, const Batch::Class& c, cudaStream_t s) {
     switch (c.G) {
+        case 64: return launch_class_fft_t<64>(b, c, s);
+        case 128: return launch_class_fft_t<128>(b, c, s);
         case 256: return launch_class_fft_t<256>(b, c, s);
         case 512: return launch_class_fft_t<512>(b, c, s);
         case 1024: return launch_class_fft_t<1024>(b, c, s);
@@ -414,6 +416,8 @@ ftcg_status_t launch_class_fft(Batch& b, const Batch::Class& c, cudaStream_t s) 
 
 std::vector<float2> class_twiddles(int G) {
     switch (G) {
+        case 64: return sfft::stage_twiddles<64>();
+        case 128: return sfft::stage_twiddles<128>();
         case 256: return sfft::stage_twiddles<256>();
         case 512: return sfft::stage_twiddles<512>();
         case 1024: return sfft::stage_twiddles<1024>();

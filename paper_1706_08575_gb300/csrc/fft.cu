@@ -8,7 +8,7 @@
 //     at most two contiguous runs of the periodic column index);
 //   * of the row transforms only the N rows of the crop are needed.
 // The other cells of the grid are left as they are (never read). The arithmetic of every kept
-// output is that of a full 2-D inverse FFT. For power-of-two G from 256 to 4096 the 1-D transforms
+// output is that of a full 2-D inverse FFT. For power-of-two G from 64 to 4096 the 1-D transforms
 // are this library's shared-memory kernels (fft_smem.cu, with the window division and crop fused
 // into the row pass); otherwise cuFFT is the 1-D engine.
 

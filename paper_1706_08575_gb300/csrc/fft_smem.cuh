@@ -1,4 +1,4 @@
-// Shared-memory 1-D FFTs of power-of-two length (256..4096) along the columns and rows of a
+// Shared-memory 1-D FFTs of power-of-two length (64..4096) along the columns and rows of a
 // G x G grid: the Stockham stages, twiddle tables and the two pass bodies used by the single-ping
 // kernels (fft_smem.cu) and the batched ones (batch.cu). See fft_smem.cu for the method.
 #pragma once
@@ -140,7 +140,7 @@ __device__ __forceinline__ void stage(float2* s, const float2* __restrict__ tw, 
     constexpr int BPT = (NB + NT - 1) / NT;
     constexpr int IN_STEP = padded(NJ);               // NJ is a multiple of 16 (or the stride is 1)
     constexpr int OUT_STEP = NS == 1 ? 1 : padded(NS);
-    static_assert(NJ % 16 == 0, "input stride must keep the padding linear");
+    static_assert(FIRST || NJ % 16 == 0, "input stride must keep the padding linear");
     static_assert(NS == 1 || NS % 16 == 0, "output stride must keep the padding linear");
     float2 v[BPT][R];
 #pragma unroll
@@ -219,7 +219,7 @@ __device__ __forceinline__ void stage_paired(float2* s, const float2* __restrict
     constexpr int PPT = (NP + NT - 1) / NT;
     constexpr int IN_STEP = padded(NJ);
     constexpr int OUT_STEP = NS == 1 ? 1 : padded(NS);
-    static_assert(NJ % 16 == 0, "input stride must keep the padding linear");
+    static_assert(FIRST || NJ % 16 == 0, "input stride must keep the padding linear");
     static_assert(NS == 1 || NS % 16 == 0, "output stride must keep the padding linear");
     float2 v[PPT][2][R];
 #pragma unroll
