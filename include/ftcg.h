@@ -153,7 +153,8 @@ ftcg_status_t ftcg_plan_info(ftcg_plan_t plan, ftcg_plan_info_t* info);
  * a gridded forward transform at 2 lambda (window width opts.weight_width).
  * The weights are installed in the plan (used by every later ftcg_adjoint) and, if d_alpha_out is
  * not NULL, written there as M float64 in acquisition order. Temporary device memory (about
- * 16 (2 sigma N)^2 bytes) is allocated and freed inside the call; the call synchronises.
+ * 12 L^2 + 72 M bytes, L the power of two from 2 sigma N up; in the FP64 route 16 (2 sigma N)^2 +
+ * 200 M) is allocated and freed inside the call; the call synchronises.
  * Errors: NUMERIC if some S_k <= 0 or is not finite (those weights are set to 0); CUDA; OOM.
  */
 ftcg_status_t ftcg_weights(ftcg_plan_t plan, double* d_alpha_out, ftcg_stream_t stream);

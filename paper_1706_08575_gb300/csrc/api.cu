@@ -41,6 +41,13 @@ namespace ftcg {
 
 void release_plan(Plan* p) {
     if (!p) return;
+    // on the plan's own device, whichever is current
+    int dev = 0;
+    cudaPointerAttributes at{};
+    const bool known = cudaGetDevice(&dev) == cudaSuccess && p->status &&
+                       cudaPointerGetAttributes(&at, p->status) == cudaSuccess &&
+                       at.type == cudaMemoryTypeDevice;
+    if (known && at.device != dev) cudaSetDevice(at.device);
     cudaDeviceSynchronize();
     free_binning(p->bin);
     // pool memory, after the synchronisation above: returned to the pool at once (cudaFree of it
@@ -62,6 +69,7 @@ void release_plan(Plan* p) {
         for (int i = 0; i < kMaxProfiled * 4; ++i) cudaEventDestroy(p->prof_ev[i]);
         delete[] p->prof_ev;
     }
+    if (known && at.device != dev) cudaSetDevice(dev);
     delete p;
 }
 
