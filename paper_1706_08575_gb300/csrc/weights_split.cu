@@ -414,10 +414,12 @@ __global__ void __launch_bounds__(kLagThreads, 2)
 // ---- transforms --------------------------------------------------------------------------------
 // Stockham stages of radix 16 (then the rest) as in fft_smem.cuh, 16 values per thread in FP32
 // pairs; exponent sign + throughout (a forward transform conjugates before and after). A CTA holds
-// 4096 values (several short lines, or one line of 8192 with twice the threads).
+// one line (two of 256, for a full warp): with 4096 values per CTA the x pass of a 20 k-sample ping
+// (L = 1024, N = 256) was 64 CTAs and the forward y pass 128, 27.6 and 19.0 us (ncu); now 26.0 and
+// 12.2.
 // Twiddles from a table of pairs, [stage][(r - 1) NS + k] = exp(2 pi i r k / (NS R)).
-__host__ __device__ constexpr int lag_lines(int L) { return L < 4096 ? 4096 / L : 1; }
-__host__ __device__ constexpr int lag_threads(int L) { return L < 4096 ? 256 : L / 16; }
+__host__ __device__ constexpr int lag_lines(int L) { return L < 512 ? 512 / L : 1; }
+__host__ __device__ constexpr int lag_threads(int L) { return L / 16 * lag_lines(L); }
 __host__ __device__ constexpr size_t lag_smem(int L) {
     return (size_t)lag_lines(L) * sfft::padded_len(L) * sizeof(float4);
 }
