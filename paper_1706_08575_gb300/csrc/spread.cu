@@ -173,8 +173,7 @@ __global__ void __launch_bounds__(kInterpThreads)
     const int e0 = colptr[(int64_t)tile * ncb] + (int)blockIdx.y * chunk;
     const int e1 = min(colptr[(int64_t)(tile + 1) * ncb], e0 + chunk);
     if (e0 >= e1) return;
-    pdl_wait();                                // the grid is complete; the next kernel is not let
-                                               // in early (its CTAs took slots: 98 -> 105 us)
+    pdl_wait();                                // the grid is complete
     // a ragged tile's samples start on its own cells only (G >= 2 w: at most one wrap)
     const int rows = min(T, G - Y0) + W - 1, cols = min(T, G - X0) + W - 1;
     for (int r = warp; r < rows; r += kInterpThreads / 32) {
