@@ -325,7 +325,9 @@ ftcg_status_t launch_interp(const Plan& p, const float2* grid, float2* vals, cud
     // after, us, w = 8, T = 32 (T = 64): N = 1024, 2.1 M samples 189, 101 (189, 120); 524 k 65, 48
     // (65, 56); 131 k at 79 per tile 33, 33; N = 256, 200 k 29, 24 (30, 28), 50 k 17, 18 (17, 21);
     // N = 500 (cuFFT), 180 k 47, 42 (47, 43), 45 k 36, 36 (36, 40).
-    if (p.M >= 98304 && b.n_entries >= (int64_t)b.T * b.T / 8 * b.n_nonempty) {
+    // A raster whose samples are all dropped has no tile to launch.
+    if (p.M >= 98304 && b.n_nonempty > 0 &&
+        b.n_entries >= (int64_t)b.T * b.T / 8 * b.n_nonempty) {
         // samples that are in no tile (not finite) read zero
         if (!b.halo || b.n_entries < p.M)
             FTCG_CK(cudaMemsetAsync(vals, 0, (size_t)p.M * sizeof(float2), s));
