@@ -69,7 +69,8 @@ __device__ __forceinline__ float sin_pi32(float x) {
 }
 
 // One axis of F_N^(1/2) for the lag dn + df (dn an integer, |dn| <= N, |df| <= 1), up to sign:
-// numerator sin(pi df), denominator sin(pi d / N); (1, 1 / N) at lag 0.
+// numerator sin(pi df), denominator sin(pi d / N); (1, 1 / N) at lag 0 and below 1e-12 (F_N differs
+// from 1 by 3e-24 there), so that no product of the two axes' factors leaves the normal FP32 range.
 __device__ __forceinline__ void fejer_axis(float dn, float df, float N, float invN, float* num,
                                            float* den) {
     if (fabsf(dn) > 0.5f * N) dn -= copysignf(N, dn);
@@ -77,8 +78,9 @@ __device__ __forceinline__ void fejer_axis(float dn, float df, float N, float in
     if (fabsf(dr) > 0.5f * N) dr -= copysignf(N, dr);    // exact (Sterbenz); now |dr| <= N/2
     const float magic = 12582912.0f;                     // 1.5 * 2^23: rounds to an integer
     const float fr = df - ((df + magic) - magic);        // sin(pi df) up to sign, |fr| <= 1/2
-    *num = dr == 0.0f ? 1.0f : sin_pi32(fr);
-    *den = dr == 0.0f ? invN : sin_pi32(dr * invN);
+    const bool zero = fabsf(dr) < 1e-12f;
+    *num = zero ? 1.0f : sin_pi32(fr);
+    *den = zero ? invN : sin_pi32(dr * invN);
 }
 
 // Block (b, p): the sums over part p of the samples of judged samples 4 b .. 4 b + 3, so that a
