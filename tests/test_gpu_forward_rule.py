@@ -3,6 +3,8 @@ density does not describe."""
 import numpy as np
 import pytest
 
+from oracle import ftcg_oracle as O
+
 pytestmark = pytest.mark.gpu
 
 
@@ -25,3 +27,20 @@ def test_all_samples_dropped(F, M, N, tile, layout):
         assert np.all(p.forward(img, out).cpu().numpy() == 0)
         x, hist, done = p.cgls(torch.ones(M, dtype=torch.complex64, device="cuda"), iters=2)
         assert np.all(x.cpu().numpy() == 0) and np.all(hist == 0) and done == 0
+
+
+@pytest.mark.parametrize("frac", [0.3, 0.5, 0.97])
+@pytest.mark.parametrize("tile,layout", [(32, 2), (64, 1)])
+def test_uneven_rasters(F, frac, tile, layout):
+    """A share of the samples in one spot, on both sides of the limit on CTAs without samples. Bar: the
+    FP32 bar of the adjoint's tests."""
+    import torch
+    M, N = 120000, 128
+    rng = np.random.default_rng(7)
+    spot = int(M * frac)
+    lam = np.concatenate([rng.random((spot, 2)) * 3.0, (rng.random((M - spot, 2)) - 0.5) * N])
+    lam = lam[rng.permutation(M)]
+    img = (rng.standard_normal((N, N)) + 1j * rng.standard_normal((N, N))).astype(np.complex64)
+    with F.Plan(torch.from_numpy(lam).cuda(), N, 2.0, 8, tile=tile, layout=layout) as p:
+        got = p.forward(torch.from_numpy(img).cuda()).cpu().numpy()
+    assert O.rel_l2(got, O.forward(lam, img.astype(np.complex128), N, 2.0, 8)) < 1e-5
