@@ -752,9 +752,8 @@ __global__ void __launch_bounds__(kLagThreads, 2)
                     const float r0 = __frcp_rn(sum.h);
                     const float e = fmaf(-sum.l, r0, fmaf(-sum.h, r0, 1.0f));
                     a = (double)r0 + (double)__fmul_rn(r0, e);
-                } else {
-                    atomicOr(bad, STATUS_BAD_WEIGHT_SUM);
-                    atomicOr(status, STATUS_BAD_WEIGHT_SUM);
+                } else if (!(atomicOr(status, STATUS_BAD_WEIGHT_SUM) & STATUS_BAD_WEIGHT_SUM)) {
+                    atomicOr(bad, STATUS_BAD_WEIGHT_SUM);      // reported once per ftcg_check
                 }
                 alpha[w.y] = a;
             }
