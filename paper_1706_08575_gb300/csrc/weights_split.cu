@@ -174,19 +174,37 @@ __device__ __forceinline__ int cell_of(unsigned w) {
     return (int)((w >> 6) & 63u) * kLagLd + (int)(w & 63u);
 }
 
+// Coordinates to positions: X = lambda 2^(46 + e) as an integer and u 2^46 = X mul / 2^64 with
+// mul = 2^64 L / (N 2^e), e such that 2^62 <= mul < 2^63.
+struct PosScale {
+    double to_x, ok, N, invN;                      // 2^(46 + e); 2 sigma (the FP64 route's scale)
+    long long mul;
+};
+inline PosScale pos_scale(int N, int L, double sigma) {
+    int extra = 0;
+    while (((long long)N << extra) <= 2ll * L) ++extra;      // mul < 2^63
+    const unsigned __int128 num = (unsigned __int128)L << 64;
+    const unsigned __int128 den = (unsigned __int128)N << extra;
+    return {std::ldexp(1.0, kFrac + extra), 2.0 * sigma, (double)N, 1.0 / N,
+            (long long)((num + den / 2) / den)};
+}
+
 // One axis: (first tap mod L) << 46 | f, or ~0 for a coordinate that is not finite or too large
-// (the same test as the FP64 route's). u = scale lambda.
-__device__ __forceinline__ unsigned long long position(double lam, double scale46, int W, int L,
-                                                       double scale_ok) {
-    double t = __dmul_rn(lam, scale46);            // u 2^46
-    // |u| >= 2^16 or not finite (exponent of t >= 62): reduce first (rare)
+// (the same test as the FP64 route's). In integers, so that u is right to a unit at every N: the
+// FP64 product with L / N, off by half an ulp of u, put the weights off by 6e-10 at N = 300 and 65536
+// periods from the origin. Far out (|lambda| >= 2^12 at L = 4 N) the whole periods are taken out
+// first, which is exact.
+__device__ __forceinline__ unsigned long long position(double lam, const PosScale& ps, int W, int L) {
+    double t = __dmul_rn(lam, ps.to_x);            // exact
     if (((unsigned)__double2hiint(t) & 0x7fffffffu) >= (1023u + 62u) << 20) {
-        const double q = __dmul_rn(lam, scale_ok);
+        const double q = __dmul_rn(lam, ps.ok);
         if (!isfinite(q) || !(fabs(q) < 1125899906842624.0)) return ~0ull;
-        const double u = t * 1.4210854715202004e-14;                         // 2^-46
-        t = (u - L * floor(u / L)) * 70368744177664.0;
+        t = __dmul_rn(fma(-ps.N, rint(__dmul_rn(lam, ps.invN)), lam), ps.to_x);
     }
-    const long long a = __double2ll_rn(t) - ((long long)W << (kFrac - 1));
+    const long long X = __double2ll_rn(t);
+    const long long u = __mul64hi(X, ps.mul) +
+                        (long long)(((unsigned long long)X * (unsigned long long)ps.mul) >> 63);
+    const long long a = u - ((long long)W << (kFrac - 1));
     const long long c = (a + (long long)kFracMask) >> kFrac;
     return ((unsigned long long)(c & (L - 1)) << kFrac) |
            (unsigned long long)((c << kFrac) - a);
@@ -195,7 +213,7 @@ __device__ __forceinline__ unsigned long long position(double lam, double scale4
 // Per sample: the two position words and its rank among the samples of its tile (in arrival
 // order, one atomic per warp and tile); the columns where taps start. Dropped samples get weight 0.
 __global__ void __launch_bounds__(256)
-    k_lag_origin(const double* __restrict__ lam, int M, double scale46, double scale_ok, int W,
+    k_lag_origin(const double* __restrict__ lam, int M, const PosScale ps, int W,
                  int L, ulonglong2* __restrict__ pos, int* __restrict__ rank,
                  int* __restrict__ cnt, unsigned char* __restrict__ first,
                  double* __restrict__ alpha, const TableArgs tables) {
@@ -210,8 +228,8 @@ __global__ void __launch_bounds__(256)
         const int64_t j = base + lane;
         int tile = -1;
         if (j < M) {
-            const unsigned long long px = position(lam[2 * j], scale46, W, L, scale_ok);
-            const unsigned long long py = position(lam[2 * j + 1], scale46, W, L, scale_ok);
+            const unsigned long long px = position(lam[2 * j], ps, W, L);
+            const unsigned long long py = position(lam[2 * j + 1], ps, W, L);
             if (px == ~0ull || py == ~0ull) {
                 alpha[j] = 0.0;
                 pos[j] = make_ulonglong2(~0ull, ~0ull);
@@ -905,9 +923,8 @@ ftcg_status_t compute_weights_split(Plan& p, double* d_alpha_out, cudaStream_t s
     const int tab = std::max(8 * kPieces * W, 2 * N);
     const TableArgs tables{W, N, (tab + 255) / 256, wa.beta, ta, tb, r2, fac};
     const int mb = std::min((M + 255) / 256, sms * 8);
-    k_lag_origin<<<tables.blocks + mb, 256, 0, s>>>(p.lambda, M, std::ldexp((double)L / N, kFrac),
-                                                    2.0 * p.sigma, W, L, pos, rank, cnt, first, alpha,
-                                                    tables);
+    k_lag_origin<<<tables.blocks + mb, 256, 0, s>>>(p.lambda, M, pos_scale(N, L, p.sigma), W, L, pos,
+                                                    rank, cnt, first, alpha, tables);
     k_lag_scan<<<1, kScanThreads, 0, s>>>(cnt, ntiles, chunk, start, items, nitems, first, W, L, occ);
     k_lag_scatter<<<mb, 256, 0, s>>>(pos, rank, M, L, start, sy, sw);
     k_lag_zero<<<L / 2, 256, 0, s>>>(grid, occ, L);
