@@ -23,9 +23,10 @@
 // sample's 2 w window values and its tap origins so that W3 reads them instead of evaluating
 // them again.
 //
-// This FP64 route serves lag grids above 8192 and windows whose truncation is below what two-float
-// arithmetic resolves (weight_width > 12, large sigma); weights_split.cu takes the others (4.97 ms
-// against about 1.1 on the large ping) and has the rule (split_lag_side).
+// This FP64 route serves what weights_split.cu does not take (split_lag_side there has the rule): lag
+// grids above 8192, windows whose truncation is below what two-float arithmetic resolves, and
+// oversamplings and widths that could be less exact on a power-of-two grid. The other is faster (large
+// ping: 4.97 ms here, about 1.1 there).
 
 #include <cuda_runtime.h>
 

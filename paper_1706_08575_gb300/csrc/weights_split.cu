@@ -849,15 +849,25 @@ struct Arena {
 
 }  // namespace
 
-// The lag grid side of this route: the power of two (256..8192) from 2 sigma N up; 0 when there is
-// none, or when the window is so wide (weight_width > 12, or exp(-beta) < 1e-13 at the plan's own
-// oversampling) that its truncation no longer covers the pairs' rounding of about 1e-14.
+// The lag grid side of this route: the power of two (256..8192) from 2 sigma N up; 0 where it is not
+// taken: without such a side, with a window so wide (weight_width > 12, or exp(-beta) < 1e-13 at the
+// plan's own oversampling) that its truncation no longer covers the pairs' rounding of about 1e-14,
+// and where the truncation could be larger than on the FP64 route's grid of side 2 sigma N. It is the
+// same on the same grid. On a finer one it is smaller on average, but varies from raster to raster by
+// more than narrow windows or a grid a few per cent finer gain (rms error against that route, polar
+// rasters: w = 4, sigma = 3 up to 5.0 times, w = 12 at sigma = 2.25, 1008 to 1024 cells, 2.7 times). The
+// default window gains for certain from a tenth more cells on (0.01 to 0.6), and at the default
+// sigma = 2 at every side measured (N = 64..1030: 0.01 to 1.03).
 int split_lag_side(const Plan& p) {
     const int W = p.opts.weight_width > 0 ? p.opts.weight_width : 12;
     if (W > kSplitMaxW || es_beta(W, p.sigma) > 29.9) return 0;
     int L = 256;
     while (L < 2 * p.G) L <<= 1;
-    return L <= 8192 ? L : 0;
+    if (L > 8192) return 0;
+    const bool same = L == 2 * p.G && p.sigma >= 2.0;
+    const bool finer = W == 12 && p.sigma >= 1.25 && p.sigma <= 2.0 &&
+                       (p.sigma == 2.0 || L >= 2.2 * p.G);
+    return same || finer ? L : 0;
 }
 
 ftcg_status_t compute_weights_split(Plan& p, double* d_alpha_out, cudaStream_t s) {

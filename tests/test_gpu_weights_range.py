@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 import sasgen
+from oracle import ftcg_oracle as O
 
 pytestmark = pytest.mark.gpu
 
@@ -31,3 +32,17 @@ def test_whole_periods_change_nothing(F, N, periods):
     lam = np.round(lam * 2.0 ** 24) / 2.0 ** 24
     ref = weights(F, lam, N)
     assert np.max(np.abs(weights(F, lam + periods * N, N) / ref - 1)) < 1e-12
+
+
+@pytest.mark.parametrize("N,sigma,wa", [
+    (256, 2.5, 4), (200, 3.0, 4), (224, 2.0, 4), (224, 2.0, 6), (224, 2.25, 12), (144, 1.75, 12),
+    (100, 2.0, 0), (300, 2.0, 0), (500, 2.0, 0), (200, 1.5, 0), (200, 1.25, 0), (128, 2.0, 4), (64, 4.0, 6),
+])
+def test_no_less_exact_than_on_the_requested_grid(F, N, sigma, wa):
+    """The rms error against pair sums is no larger than that of the FP64 lag route on a grid of side
+    2 sigma N, whatever grid the library takes. 10 % and 1e-13 for the two routes' rounding."""
+    lam = sasgen.random_case(N + wa, 1500, N, spread=N)[0]
+    ref, _ = O.weights_brute(lam, N)
+    err = lambda a: np.sqrt(np.mean((a / ref - 1) ** 2))
+    assert err(weights(F, lam, N, sigma, wa)) < \
+        1.1 * err(O.weights_nufft(lam, N, sigma, wa or 12)[0]) + 1e-13
