@@ -397,7 +397,7 @@ Win32 win32_of(const Window& win);
 ftcg_status_t compute_weights(Plan& p, double* d_alpha_out, cudaStream_t s);
 // weights_split.cu: the same without the FP64 pipe; the lag grid side it would use (0: not taken)
 int split_lag_side(const Plan& p);
-ftcg_status_t compute_weights_split(Plan& p, double* d_alpha_out, cudaStream_t s);
+ftcg_status_t compute_weights_split(Plan& p, double* d_alpha_out, cudaStream_t s, bool* uneven);
 // judge.cu: exact Fejer sums at K samples, the verdict, and its installation
 ftcg_status_t judge_launch(const Plan& p, const double* d_alpha, int K, double* d_S, double* d_a,
                            cudaStream_t s);

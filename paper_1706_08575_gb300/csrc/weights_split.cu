@@ -643,11 +643,14 @@ __global__ void __launch_bounds__(lag_threads(L), 65536 / 128 / lag_threads(L))
 }
 
 // Along x, rows m = 0..N-1 of spec: forward, times the lag weights, back (one loop, for the
-// instruction cache); only occupied columns are read (the others are zero) and written.
+// instruction cache); only occupied columns are read (the others are zero) and written. energy: the
+// kEnergy partial sums of |coefficient|^2 over all frequencies, which is the mean square of the S grid.
+constexpr int kEnergy = 32;
 template <int L>
 __global__ void __launch_bounds__(lag_threads(L), 65536 / 128 / lag_threads(L))
     k_lag_fft_x(float4* __restrict__ spec, int N, const unsigned char* __restrict__ occ,
-                const float4* __restrict__ tw, const float2* __restrict__ fac) {
+                const float4* __restrict__ tw, const float2* __restrict__ fac,
+                double* __restrict__ energy) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int LINES = lag_lines(L), TL = L / 16;
     const int line = threadIdx.x / TL, t = threadIdx.x - line * TL;
@@ -668,6 +671,7 @@ __global__ void __launch_bounds__(lag_threads(L), 65536 / 128 / lag_threads(L))
     for (int pass = 0; pass < 2; ++pass) {
         lag_transform<L>(u, sm, tw, t);
         if (pass == 0) {
+            float sq = 0.f;
 #pragma unroll
             for (int r = 0; r < 16; ++r) {
                 const int q = t + r * TL;
@@ -676,10 +680,14 @@ __global__ void __launch_bounds__(lag_threads(L), 65536 / 128 / lag_threads(L))
                     const float2 g = fac[i];
                     const ff f = fy * ff{g.x, g.y};
                     u[r] = {u[r].x * f, -(u[r].y * f)};
+                    sq = fmaf(u[r].x.h, u[r].x.h, fmaf(u[r].y.h, u[r].y.h, sq));
                 } else {
                     u[r] = {{0.f, 0.f}, {0.f, 0.f}};
                 }
             }
+            if (m > 0) sq += sq;                   // row -m
+            for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+            if ((threadIdx.x & 31) == 0) atomicAdd(energy + blockIdx.x % kEnergy, (double)sq);
         }
     }
     if (!on) return;
@@ -695,6 +703,14 @@ __global__ void __launch_bounds__(lag_threads(L), 65536 / 128 / lag_threads(L))
 // sample; lane q holds taps q, q + 4, q + 8 of both axes, sums its columns over the x taps (shuffled)
 // and weights them; alpha = 1 / S by one Newton step on the FP32 reciprocal. Bound: instruction issue
 // (12 FP32 operations per tap). Large ping: 888 us in FP64 from global memory, here 306 us.
+//
+// The transforms' rounding is relative to the whole raster: it puts an S_k off by 1.1e-14 (rms) of the
+// S grid's root mean square. A sample alone next to a dense cluster sees that as a larger relative error
+// than the window's truncation once rms / S_k is above some 100 (N = 512: 1.2 times the error of the FP64
+// route at 128..256, 1.9 at 256..1024; with 4 M samples in one spot 13 times). From kUneven on the raster is
+// left to the FP64 route, whose rounding does not show. A polar raster reaches 11 (2 M samples, N = 256).
+constexpr float kUneven = 64.0f;
+constexpr unsigned kBadSum = 1u, kTooUneven = 2u;
 struct InterpSmem {
     float4 ta[kPieces * kSplitMaxW], tb[kPieces * kSplitMaxW];
     float2 g[kLagCells];
@@ -707,6 +723,7 @@ __global__ void __launch_bounds__(kLagThreads, 2)
                  const int4* __restrict__ items, const int* __restrict__ nitems,
                  int* __restrict__ next, const float4* __restrict__ ta,
                  const float4* __restrict__ tb, int w_arg, int L, const float2* __restrict__ grid,
+                 const double* __restrict__ energy, const float2* __restrict__ fac, int N,
                  double* __restrict__ alpha, unsigned* __restrict__ bad,
                  unsigned* __restrict__ status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -718,11 +735,17 @@ __global__ void __launch_bounds__(kLagThreads, 2)
     }
     const int q = threadIdx.x & 3, nt = L / kLagTile, ni = *nitems;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    static_assert(kEnergy == 32, "one lane per partial sum");
+    double ms = energy[lane];
+    for (int o = 16; o > 0; o >>= 1) ms += __shfl_xor_sync(0xffffffffu, ms, o);
+    // S_k is a window's sum over the grid: 1 / r(0)^2 = 1 / (N fac[m = 0]) times its cells
+    const float least = sqrtf((float)ms) / ((float)N * fac[N].x * kUneven);
+    bool uneven = false;
     for (;;) {
         __syncthreads();                           // tables staged; the last tile consumed
         if (threadIdx.x == 0) s.item = atomicAdd(next, 1);
         __syncthreads();
-        if (s.item >= ni) return;
+        if (s.item >= ni) break;
         const int4 item = items[s.item];
         const int X0 = item.x / nt * kLagTile, Y0 = item.x % nt * kLagTile;
         for (int r = warp; r < kLagTile + W - 1; r += kLagWarps) {   // every y of those columns
@@ -766,17 +789,20 @@ __global__ void __launch_bounds__(kLagThreads, 2)
             if (q == 0 && on) {
                 sum = norm(sum);
                 double a = 0.0;
-                if (sum.h > 0.0f && isfinite(sum.h)) {
+                if (sum.h < least) {
+                    uneven = true;
+                } else if (sum.h > 0.0f && isfinite(sum.h)) {
                     const float r0 = __frcp_rn(sum.h);
                     const float e = fmaf(-sum.l, r0, fmaf(-sum.h, r0, 1.0f));
                     a = (double)r0 + (double)__fmul_rn(r0, e);
                 } else if (!(atomicOr(status, STATUS_BAD_WEIGHT_SUM) & STATUS_BAD_WEIGHT_SUM)) {
-                    atomicOr(bad, STATUS_BAD_WEIGHT_SUM);      // reported once per ftcg_check
+                    atomicOr(bad, kBadSum);        // reported once per ftcg_check
                 }
                 alpha[w.y] = a;
             }
         }
     }
+    if (uneven) atomicOr(bad, kTooUneven);
 }
 
 // ---- host ------------------------------------------------------------------------------------
@@ -818,14 +844,14 @@ ftcg_status_t lag_twiddles(int L, cudaStream_t s, const float4** out) {
 
 template <int L>
 ftcg_status_t lag_transforms(double* grid, float4* spec, int N, const unsigned char* occ,
-                             const float2* fac, const float4* tw, cudaStream_t s) {
+                             const float2* fac, const float4* tw, double* energy, cudaStream_t s) {
     constexpr int NT = lag_threads(L), LINES = lag_lines(L);
     const int sm = (int)lag_smem(L);
     FTCG_CK(cudaFuncSetAttribute(k_lag_fft_y<L, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
     FTCG_CK(cudaFuncSetAttribute(k_lag_fft_y<L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
     FTCG_CK(cudaFuncSetAttribute(k_lag_fft_x<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
     k_lag_fft_y<L, false><<<L / 2 / LINES, NT, sm, s>>>(grid, spec, N, occ, tw);
-    k_lag_fft_x<L><<<(N + LINES - 1) / LINES, NT, sm, s>>>(spec, N, occ, tw, fac);
+    k_lag_fft_x<L><<<(N + LINES - 1) / LINES, NT, sm, s>>>(spec, N, occ, tw, fac, energy);
     k_lag_fft_y<L, true><<<L / 2 / LINES, NT, sm, s>>>(grid, spec, N, occ, tw);
     FTCG_CK(cudaGetLastError());
     return FTCG_SUCCESS;
@@ -870,7 +896,9 @@ int split_lag_side(const Plan& p) {
     return same || finer ? L : 0;
 }
 
-ftcg_status_t compute_weights_split(Plan& p, double* d_alpha_out, cudaStream_t s) {
+// *uneven: the raster is left to the FP64 route (see kUneven); its weights here don't count.
+ftcg_status_t compute_weights_split(Plan& p, double* d_alpha_out, cudaStream_t s, bool* uneven) {
+    *uneven = false;
     const int W = p.opts.weight_width > 0 ? p.opts.weight_width : 12;
     const int L = split_lag_side(p), N = p.N, M = (int)p.M;
     const Window wa{W, es_beta(W, (double)L / (2.0 * N))};
@@ -885,7 +913,7 @@ ftcg_status_t compute_weights_split(Plan& p, double* d_alpha_out, cudaStream_t s
     const int max_items = std::min(ntiles, M) + M / chunk;
     Arena ar;
     ar.s = s;
-    double *r2, *grid, *alpha;
+    double *r2, *grid, *alpha, *energy;
     float4 *ta, *tb, *spec;
     float2* fac;
     ulonglong2* pos;
@@ -898,10 +926,11 @@ ftcg_status_t compute_weights_split(Plan& p, double* d_alpha_out, cudaStream_t s
     size_t zero_bytes = 0;
     auto lay_out = [&]() {
         ar.used = 0;
-        cnt = ar.take<int>(ntiles);                // cleared together, up to next
+        cnt = ar.take<int>(ntiles);                // cleared together, up to energy
         first = ar.take<unsigned char>(L);
         bad = ar.take<unsigned>(1);
         next = ar.take<int>(2);                    // item counters of W1 and W3
+        energy = ar.take<double>(kEnergy);
         zero_bytes = ar.used;
         r2 = ar.take<double>(2 * (size_t)N);
         fac = ar.take<float2>(2 * (size_t)N);
@@ -949,22 +978,23 @@ ftcg_status_t compute_weights_split(Plan& p, double* d_alpha_out, cudaStream_t s
                                                          grid);
     FTCG_CK(cudaGetLastError());
     switch (L) {
-        case 256: FTCG_TRY(lag_transforms<256>(grid, spec, N, occ, fac, tw, s)); break;
-        case 512: FTCG_TRY(lag_transforms<512>(grid, spec, N, occ, fac, tw, s)); break;
-        case 1024: FTCG_TRY(lag_transforms<1024>(grid, spec, N, occ, fac, tw, s)); break;
-        case 2048: FTCG_TRY(lag_transforms<2048>(grid, spec, N, occ, fac, tw, s)); break;
-        case 4096: FTCG_TRY(lag_transforms<4096>(grid, spec, N, occ, fac, tw, s)); break;
-        default: FTCG_TRY(lag_transforms<8192>(grid, spec, N, occ, fac, tw, s)); break;
+        case 256: FTCG_TRY(lag_transforms<256>(grid, spec, N, occ, fac, tw, energy, s)); break;
+        case 512: FTCG_TRY(lag_transforms<512>(grid, spec, N, occ, fac, tw, energy, s)); break;
+        case 1024: FTCG_TRY(lag_transforms<1024>(grid, spec, N, occ, fac, tw, energy, s)); break;
+        case 2048: FTCG_TRY(lag_transforms<2048>(grid, spec, N, occ, fac, tw, energy, s)); break;
+        case 4096: FTCG_TRY(lag_transforms<4096>(grid, spec, N, occ, fac, tw, energy, s)); break;
+        default: FTCG_TRY(lag_transforms<8192>(grid, spec, N, occ, fac, tw, energy, s)); break;
     }
     interp<<<ctas, kLagThreads, sizeof(InterpSmem), s>>>(
-        sy, sw, items, nitems, next + 1, ta, tb, W, L, reinterpret_cast<const float2*>(grid), alpha,
-        bad, p.status);
+        sy, sw, items, nitems, next + 1, ta, tb, W, L, reinterpret_cast<const float2*>(grid), energy,
+        fac, N, alpha, bad, p.status);
     FTCG_CK(cudaGetLastError());
     FTCG_TRY(launch_set_alpha(p, alpha, FTCG_WEIGHTS_F64, s));
     unsigned seen = 0;
     FTCG_CK(cudaMemcpyAsync(&seen, bad, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
     FTCG_CK(cudaStreamSynchronize(s));
-    if (seen) {
+    *uneven = (seen & kTooUneven) != 0;
+    if (seen & kBadSum) {
         set_error("ftcg_weights: a weight sum S_k was <= 0 or not finite (weight set to 0)");
         return FTCG_ERR_NUMERIC;
     }

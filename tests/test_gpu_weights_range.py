@@ -46,3 +46,23 @@ def test_no_less_exact_than_on_the_requested_grid(F, N, sigma, wa):
     err = lambda a: np.sqrt(np.mean((a / ref - 1) ** 2))
     assert err(weights(F, lam, N, sigma, wa)) < \
         1.1 * err(O.weights_nufft(lam, N, sigma, wa or 12)[0]) + 1e-13
+
+
+@pytest.mark.parametrize("N", [512, 1000])
+def test_samples_alone_next_to_a_cluster(F, N):
+    """300 samples alone in the plane, four million in one spot: the lone samples' S_k are about 1, next to
+    4e6 in the cluster. Against pair sums in FP64. Bar: that of test_gpu_weights_split."""
+    import torch
+    M = 4000000
+    rng = np.random.default_rng(N)
+    lam = np.concatenate([(rng.random((300, 2)) - 0.5) * N,
+                          0.3 + 0.1 * rng.standard_normal((M - 300, 2))])
+    k = np.r_[0:300, 300:M:M // 20]
+    x, S = torch.from_numpy(lam).cuda(), []
+    for c in k:
+        d = x - x[c]
+        d -= N * torch.round(d / N)
+        f = torch.sin(np.pi * (d - torch.round(d))) / (N * torch.sin(np.pi * d / N))
+        S.append(torch.where(d == 0, torch.ones_like(d), f).square().prod(1).sum().item())
+    tol = 100 * np.exp(-0.97 * np.pi * 0.75 * 12) + 1e-12
+    assert np.max(np.abs(weights(F, lam, N)[k] * S - 1)) < tol
