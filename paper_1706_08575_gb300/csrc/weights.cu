@@ -427,7 +427,9 @@ ftcg_status_t compute_weights(Plan& p, double* d_alpha_out, cudaStream_t s) {
     if (split_lag_side(p) > 0) {
         bool uneven = false;
         const ftcg_status_t st = compute_weights_split(p, d_alpha_out, s, &uneven);
-        if (!uneven) return st;
+        // without memory for its lag grid: the one below can be up to four times smaller
+        if (!uneven && st != FTCG_ERR_OUT_OF_MEMORY) return st;
+        clear_error();
     }
     const int Wa = p.opts.weight_width > 0 ? p.opts.weight_width : 12;
     const int N2 = 2 * p.N;

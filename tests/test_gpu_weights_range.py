@@ -1,5 +1,9 @@
 """Exact weights of rasters that the usual ones do not describe: far from the origin, strongly uneven,
 window widths and oversamplings whose lag grid is no power of two."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -7,6 +11,7 @@ import sasgen
 from oracle import ftcg_oracle as O
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
@@ -66,3 +71,21 @@ def test_samples_alone_next_to_a_cluster(F, N):
         S.append(torch.where(d == 0, torch.ones_like(d), f).square().prod(1).sum().item())
     tol = 100 * np.exp(-0.97 * np.pi * 0.75 * 12) + 1e-12
     assert np.max(np.abs(weights(F, lam, N)[k] * S - 1)) < tol
+
+
+def test_little_device_memory(F):
+    """N = 1030 with 600 MiB free: too little for the lag grid of side 8192 (672 MB), enough for the one of
+    2 sigma N = 4120 (272 MB). In a process of its own, whose memory pool is empty."""
+    code = """
+import numpy as np, torch
+import paper_1706_08575_gb300 as F, sasgen
+from oracle import ftcg_oracle as O
+lam = sasgen.random_case(3, 300, 1030, spread=60)[0]
+with F.Plan(torch.from_numpy(lam).cuda(), 1030, 2.0, 6) as p:
+    torch.cuda.synchronize()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (600 << 20), dtype=torch.uint8, device="cuda")
+    a = p.weights().cpu().numpy()
+assert np.max(np.abs(a / O.weights_brute(lam, 1030)[0] - 1)) < 1e-10
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
