@@ -97,8 +97,13 @@ __device__ __forceinline__ void rho_axis(double xj, double sj, double cj, double
     const double t = fma(d, invN, magic), dr = fma(-(t - magic), N, d);
     double n = fma(sj, ca, -(cj * sa));
     double e = N * sin_pi(dr * invN);
-    if (fabs(dr) < 0.5) n = dr == 0.0 ? 1.0 : sin_pi(dr);
-    if (dr == 0.0) e = 1.0;
+    // compared by the exponent bits, off the FP64 pipe
+    const unsigned hi = (unsigned)__double2hiint(dr) & 0x7fffffffu;
+    // lag 0, and below 2^-332 (rho differs from 1 by 1e-199 there), so that the product of the two
+    // axes' factors stays a normal number
+    const bool zero = hi < (1023u - 332u) << 20;
+    if (hi < (1023u - 1u) << 20) n = zero ? 1.0 : sin_pi(dr);        // |dr| < 1/2
+    if (zero) e = 1.0;
     *num = n;
     *den = __double2loint(t) & 1 ? -e : e;
 }
