@@ -109,8 +109,11 @@ __device__ __forceinline__ void rho_axis(double xj, double sj, double cj, double
 }
 
 // rho over the upper tile pairs: CTA (tile row, tile column >= tile row) of 32 x 32 entries,
-// written as they are and transposed.
+// written as they are and transposed. While the tiles leave SMs idle, Z = 4 CTAs take 8 rows of a
+// tile each: an entry is about 60 FP64 instructions, so that a whole tile is 15 us of one SM's pipe.
+// Whole call at M = 100, r = 1, us: one thread per entry 101, tiles by one CTA 117, by four 97.
 constexpr int kGramTile = 32;
+template <int Z>
 __global__ void __launch_bounds__(256)
     k_gram(const BandSample* __restrict__ smp, int M, int N, double* __restrict__ rho) {
     if (blockIdx.x < blockIdx.y) return;
@@ -127,7 +130,7 @@ __global__ void __launch_bounds__(256)
     const double Nd = (double)N, invN = 1.0 / N;
     const int jj = threadIdx.x & 31, ar = threadIdx.x >> 5;
     const double* q = sj[jj];
-    for (int ai = ar; ai < kGramTile; ai += 8) {
+    for (int ai = ar + (Z > 1 ? 8 * blockIdx.z : 0); ai < kGramTile; ai += 8 * Z) {
         const double* p = sa[ai];
         double nx, dx, ny, dy;
         rho_axis(q[0], q[1], q[2], p[0], p[1], p[2], Nd, invN, &nx, &dx);
@@ -138,6 +141,7 @@ __global__ void __launch_bounds__(256)
     }
     if (blockIdx.x == blockIdx.y) return;
     __syncthreads();
+    if (Z > 1 && (jj >> 3) % Z != blockIdx.z) return;      // the rows of this CTA
     for (int ji = ar; ji < kGramTile; ji += 8)
         if (j0 + ji < M && a0 + jj < M) rho[(int64_t)(j0 + ji) * M + a0 + jj] = out[jj][ji];
 }
@@ -145,7 +149,9 @@ __global__ void __launch_bounds__(256)
 // G2[a * nb + o] = (rho^2)_{a, a+o} = sum_j rho_aj rho_{a+o,j}, o = 0..nb-1 (0 past the last
 // sample). A CTA takes the ar nb <= 256 entries of ar rows, one per thread; the ar + nb - 1 rows
 // are staged 64 columns at a time, so that each is read about twice instead of 2 nb times, and a
-// thread adds the sums of 64 terms (blocked summation).
+// thread adds the sums of 64 terms (blocked summation). The rows per CTA are such that a small M
+// occupies the GPU too: with as many as fit, M = 100, r = 1 ran on two SMs (whole call 120 us; one warp
+// per entry 103).
 constexpr int kG2Cols = 64, kG2MaxRows = 64;
 __global__ void __launch_bounds__(256)
     k_gram2_band(const double* __restrict__ rho, int M, int nb, int ar, double* __restrict__ G2) {
@@ -163,10 +169,12 @@ __global__ void __launch_bounds__(256)
         __syncthreads();
         if (on) {
             const double *p = sm_g2 + ia * ld, *q = p + o * ld;
-            double part = 0.0;
-#pragma unroll 8
-            for (int c = 0; c < kG2Cols; ++c) part = fma(p[c], q[c], part);
-            sum += part;
+            double part[4] = {0.0, 0.0, 0.0, 0.0};     // four chains in flight
+#pragma unroll 4
+            for (int c = 0; c < kG2Cols; c += 4)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) part[k] = fma(p[c + k], q[c + k], part[k]);
+            sum += (part[0] + part[1]) + (part[2] + part[3]);
         }
     }
     if (on) G2[(int64_t)(a0 + ia) * nb + o] = sum;
@@ -309,20 +317,26 @@ extern "C" ftcg_status_t ftcg_band(ftcg_plan_t plan, int32_t r, void* d_coef_out
     release_band(p);
     if (M == 0) return FTCG_SUCCESS;
     const int nc = 2 * r - 1, nb = 2 * r - 1;      // unknowns per column, offsets of T^2
-    double *rho = nullptr, *G2 = nullptr;
-    BandSample* smp = nullptr;
+    BandSample* smp = nullptr;                     // then rho and G2: one allocation
     cd* C = nullptr;
-    FTCG_CK(pool_malloc(&rho, (size_t)M * M * sizeof(double), s));
-    FTCG_CK(pool_malloc(&G2, (size_t)M * nb * sizeof(double), s));
-    FTCG_CK(pool_malloc(&smp, (size_t)M * sizeof(BandSample), s));
+    FTCG_CK(pool_malloc(&smp, (size_t)M * sizeof(BandSample) +
+                                  ((size_t)M * M + (size_t)M * nb) * sizeof(double), s));
+    double* rho = reinterpret_cast<double*>(smp + M);
+    double* G2 = rho + (size_t)M * M;
     FTCG_CK(pool_malloc(&C, (size_t)M * nc * sizeof(cd), s));
     p->band_c = C;
     FTCG_CK(pool_malloc(&p->band_tau, (size_t)M * sizeof(float2), s));
     p->band_r = r;
     k_band_prep<<<(M + 127) / 128, 128, 0, s>>>(p->lambda, M, p->N, smp);
     const int nt = (M + kGramTile - 1) / kGramTile;
-    k_gram<<<dim3(nt, nt), 256, 0, s>>>(smp, M, p->N, rho);
-    const int ar = std::min(kG2MaxRows, 256 / nb);
+    int dev = 0, sms = 0;
+    FTCG_CK(cudaGetDevice(&dev));
+    FTCG_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (nt * (nt + 1) / 2 < sms)
+        k_gram<4><<<dim3(nt, nt, 4), 256, 0, s>>>(smp, M, p->N, rho);
+    else
+        k_gram<1><<<dim3(nt, nt), 256, 0, s>>>(smp, M, p->N, rho);
+    const int ar = std::min(std::min(kG2MaxRows, 256 / nb), std::max(4, (M + sms - 1) / sms));
     k_gram2_band<<<(M + ar - 1) / ar, 256, (size_t)(ar + nb - 1) * (kG2Cols + 1) * sizeof(double),
                    s>>>(rho, M, nb, ar, G2);
     const size_t sm = (size_t)kSolveCols * packed_len(nc) * sizeof(double);
@@ -332,8 +346,6 @@ extern "C" ftcg_status_t ftcg_band(ftcg_plan_t plan, int32_t r, void* d_coef_out
     if (d_coef_out)
         FTCG_CK(cudaMemcpyAsync(d_coef_out, C, (size_t)M * nc * sizeof(cd),
                                 cudaMemcpyDeviceToDevice, s));
-    FTCG_CK(pool_free(rho, s));
-    FTCG_CK(pool_free(G2, s));
     FTCG_CK(pool_free(smp, s));
     // C replaces the diagonal weights: spread tau = C v with unit weights
     FTCG_TRY(launch_set_alpha(*p, nullptr, FTCG_WEIGHTS_F64, s));
