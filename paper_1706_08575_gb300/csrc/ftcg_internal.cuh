@@ -165,6 +165,7 @@ struct Binning {
     int G = 0, T = 0, W = 0;
     int ntx = 0, ntiles = 0, ncb = 0;   // ncb = T + W - 1 column bins per tile
     int64_t n_entries = 0;
+    bool dropped = false;               // some samples have no entry (non-finite coordinates)
     Entry* ent = nullptr;               // n_entries, sorted by (tile, column bin, row)
     int* colptr = nullptr;              // ntiles * ncb + 1 start offsets
     int* tile_order = nullptr;          // tiles by decreasing entry count (launch order)

@@ -474,6 +474,7 @@ ftcg_status_t build_binning(Binning& b, const double* d_lambda, int64_t M, doubl
         FTCG_CK(cudaStreamSynchronize(s));
         b.n_entries = h[0];
         *status = (unsigned)h[1];
+        b.dropped = (*status & STATUS_NONFINITE_COORD) != 0;
         b.tile_cnt.assign(h.begin() + kSumHead, h.begin() + kSumHead + b.ntiles);
         FTCG_TRY(order_tiles(b, reinterpret_cast<unsigned char*>(h.data() + kSumHead + b.ntiles), s,
                              bytes));

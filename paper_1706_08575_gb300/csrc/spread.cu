@@ -320,8 +320,8 @@ ftcg_status_t launch_pad_apod(const Plan& p, const float2* img, float2* grid, cu
 static ftcg_status_t launch_interp_tiles(const Plan& p, const float2* grid, float2* vals,
                                          const Win32& win, int chunk, int parts, cudaStream_t s) {
     const Binning& b = p.bin;
-    // samples that are in no tile (not finite) read zero
-    if (!b.halo || b.n_entries < p.M)
+    // samples that are in no tile read zero
+    if (b.dropped)
         FTCG_CK(cudaMemsetAsync(vals, 0, (size_t)p.M * sizeof(float2), s));
     const int side = b.T + b.W - 1;
     const size_t sm = (size_t)side * (side | 1) * sizeof(float2);
@@ -342,9 +342,15 @@ ftcg_status_t launch_interp(const Plan& p, const float2* grid, float2* vals, cud
     // after, us, w = 8, T = 32 (T = 64): N = 1024, 2.1 M samples 189, 101 (189, 120); 524 k 65, 48
     // (65, 56); 131 k at 79 per tile 33, 33; N = 256, 200 k 29, 24 (30, 28), 50 k 17, 18 (17, 21);
     // N = 500 (cuFFT), 180 k 47, 42 (47, 43), 45 k 36, 36 (36, 40).
+    // In the duplicate layout a tile also visits samples that are another tile's. Wide windows pay later
+    // there (w = 16, N = 256, T = 64: 130 k 64, 67, 300 k 110, 98), and narrow ones in tiles of 64 only
+    // from 5/4 entries per cell on (w = 8: N = 500, 200 k 55, 59, N = 256, 200 k 48, 42); w = 9..12 and
+    // T = 32 as in the halo layout (w = 8, N = 500, 200 k 55, 55; w = 10, 76, 64).
     // A raster whose samples are all dropped has no tile to launch.
-    if (p.M >= 98304 && b.n_nonempty > 0 &&
-        b.n_entries >= (int64_t)b.T * b.T / 8 * b.n_nonempty) {
+    const int64_t cells = (int64_t)b.T * b.T * b.n_nonempty;
+    const int64_t least = !b.halo && p.w > 12 ? 262144 : 98304;
+    if (p.M >= least && b.n_nonempty > 0 &&
+        b.n_entries >= (!b.halo && p.w <= 8 && b.T == 64 ? cells / 4 * 5 : cells / 8)) {
         // parts of 256 to 1024 samples: eight CTAs per SM where the raster allows it
         int dev = 0, sms = 0;
         FTCG_CK(cudaGetDevice(&dev));

@@ -44,3 +44,25 @@ def test_uneven_rasters(F, frac, tile, layout):
     with F.Plan(torch.from_numpy(lam).cuda(), N, 2.0, 8, tile=tile, layout=layout) as p:
         got = p.forward(torch.from_numpy(img).cuda()).cpu().numpy()
     assert O.rel_l2(got, O.forward(lam, img.astype(np.complex128), N, 2.0, 8)) < 1e-5
+
+
+@pytest.mark.parametrize("M,N,w,tile,drop", [
+    (262144, 90, 16, 64, 0), (262143, 90, 16, 64, 2), (270001, 100, 13, 32, 3),      # wide windows
+    (120000, 128, 8, 64, 0), (120000, 250, 8, 64, 4), (120000, 250, 5, 32, 0), (100000, 128, 12, 64, 1),
+])
+def test_duplicate_layout(F, M, N, w, tile, drop):
+    """Every sample written once by the tile of its first tap, dropped ones read zero, on both sides of
+    the duplicate layout's lines. Bar: the FP32 bar of the adjoint's tests."""
+    import torch
+    rng = np.random.default_rng(M + N)
+    lam = (rng.random((M, 2)) - 0.5) * N
+    img = (rng.standard_normal((N, N)) + 1j * rng.standard_normal((N, N))).astype(np.complex64)
+    bad = rng.choice(M, drop, replace=False)
+    lam[bad] = np.inf
+    with F.Plan(torch.from_numpy(lam).cuda(), N, 2.0, w, tile=tile, layout=1, allow_numeric=True) as p:
+        out = torch.full((M,), 7.0 + 0j, dtype=torch.complex64, device="cuda")
+        got = p.forward(torch.from_numpy(img).cuda(), out).cpu().numpy()
+    keep = np.ones(M, bool)
+    keep[bad] = False
+    assert O.rel_l2(got[keep], O.forward(lam[keep], img.astype(np.complex128), N, 2.0, w)) < 1e-5
+    assert np.all(got[bad] == 0)
