@@ -89,3 +89,22 @@ assert np.max(np.abs(a / O.weights_brute(lam, 1030)[0] - 1)) < 1e-10
 """
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr
+
+
+@pytest.mark.parametrize("N", [130, 200, 256])
+def test_against_pair_sums_at_lag_side_1024(F, N):
+    """Bar of test_gpu_weights_split, which has the other lag grid sides."""
+    lam = sasgen.random_case(N, 1500, N, spread=60)[0]
+    ref, _ = O.weights_brute(lam, N)
+    assert np.max(np.abs(weights(F, lam, N) / ref - 1)) < 100 * np.exp(-0.97 * np.pi * 9.0) + 1e-12
+
+
+def test_full_accumulators(F):
+    """640,000 samples on four lattice points: work items of 1023 samples (from 622 k samples on), each of
+    which adds the largest product, 1, to one cell. The lattice points don't see one another, so a weight is
+    one over its point's multiplicity."""
+    n = np.array([1023, 200000, 318977, 120000])
+    pts = np.array([[0.0, 0.0], [3.0, -7.0], [-20.0, 11.0], [31.0, 30.0]])
+    which = np.random.default_rng(1).permutation(np.repeat(np.arange(4), n))
+    a = weights(F, pts[which], 64)
+    assert np.max(np.abs(a * n[which] - 1)) < 100 * np.exp(-0.97 * np.pi * 9.0) + 1e-12
