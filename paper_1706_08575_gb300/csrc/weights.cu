@@ -429,6 +429,7 @@ ftcg_status_t compute_weights(Plan& p, double* d_alpha_out, cudaStream_t s) {
         const ftcg_status_t st = compute_weights_split(p, d_alpha_out, s, &uneven);
         // without memory for its lag grid: the one below can be up to four times smaller
         if (!uneven && st != FTCG_ERR_OUT_OF_MEMORY) return st;
+        if (st != FTCG_SUCCESS) cudaGetLastError();
         clear_error();
     }
     const int Wa = p.opts.weight_width > 0 ? p.opts.weight_width : 12;
