@@ -90,7 +90,7 @@ typedef struct {
     int32_t kernel;        /* FTCG_WINDOW_ES (default), _KB or _GAUSS                          */
     int32_t precision;     /* FTCG_PREC_FP32 (default) or FTCG_PREC_BF16 weight storage        */
     int32_t tile;          /* fine-grid tile side of the spreading kernel: 0 = auto, 32 or 64 */
-    int32_t weight_width;  /* window width of the FP64 weight construction: 0 = 12, else 4..16 */
+    int32_t weight_width;  /* window width of the weight construction: 0 = 12, else 4..16      */
     int32_t layout;        /* FTCG_LAYOUT_AUTO (default), _DUPLICATE or _HALO                  */
     int32_t spread_kernel; /* FTCG_SPREAD_AUTO (default), _WINDOW, _TENSOR or _BLOCK            */
     int32_t deterministic; /* 1: adjoints bitwise reproducible (see below); 0 (default): fastest */
@@ -103,8 +103,8 @@ typedef struct {
  * cell in a fixed order (left, upper-left, upper neighbour) instead of by atomics. Two plans
  * built from the same inputs then give bitwise equal adjoints (one warp per tile: the large ping's
  * spreading stage takes 203 us against 76 us). Needs what the block kernel needs (w <= 8, see FTCG_SPREAD_BLOCK) and G = sigma N a
- * multiple of the tile side; FTCG_ERR_NOT_SUPPORTED otherwise, and for batches. The FP64
- * weights of ftcg_weights are not covered (their first step sums with atomics). */
+ * multiple of the tile side; FTCG_ERR_NOT_SUPPORTED otherwise, and for batches. The weights of
+ * ftcg_weights are not covered (their first step sums with FP64 atomics). */
 
 typedef struct {
     int64_t M;             /* samples                                                           */
@@ -147,14 +147,17 @@ ftcg_status_t ftcg_plan_info(ftcg_plan_t plan, ftcg_plan_info_t* info);
  *     S_k = sum_j F_N(lambda_jx - lambda_kx) F_N(lambda_jy - lambda_ky),
  *     F_N(d) = sin^2(pi d) / (N^2 sin^2(pi d / N))   (normalised Fejer kernel),
  * i.e. the column-wise least-squares optimum of || T D - I ||_F with T the data-frame Gram matrix
- * on the N x N pixel lattice. Computed on the device by the lag route, in FP64 or in FP32 pairs and
- * 64-bit integers where the window's truncation is larger than their rounding (same error): a gridded adjoint
- * of unit strengths at 2 lambda on a 2N lattice, a product with c(d) = prod (N - |d_i|) / N^2, and
- * a gridded forward transform at 2 lambda (window width opts.weight_width).
+ * on the N x N pixel lattice. Computed on the device by the lag route: a gridded adjoint of unit
+ * strengths at 2 lambda on a 2N lattice, a product with c(d) = prod (N - |d_i|) / N^2, and a gridded
+ * forward transform at 2 lambda (window width opts.weight_width). In FP64, or in FP32 pairs and 64-bit
+ * integers where that is no less exact: the default width at sigma = 2 (or on a lag grid a tenth finer
+ * than 2 sigma N, sigma 1.25..2) and any width up to 12 on the grid 2 sigma N itself, unless some S_k is
+ * below 1/64 of the root mean square of S over the period (a sample alone next to a dense cluster),
+ * which is found out on the way and costs that time.
  * The weights are installed in the plan (used by every later ftcg_adjoint) and, if d_alpha_out is
  * not NULL, written there as M float64 in acquisition order. Temporary device memory (about
- * 12 L^2 + 72 M bytes, L the power of two from 2 sigma N up; in the FP64 route 16 (2 sigma N)^2 +
- * 200 M) is allocated and freed inside the call; the call synchronises.
+ * 12 L^2 + 72 M bytes, L the power of two from 2 sigma N up; without them, and in the FP64 route, 16 (2
+ * sigma N)^2 + 200 M) is allocated and freed inside the call; the call synchronises.
  * Errors: NUMERIC if some S_k <= 0 or is not finite (those weights are set to 0); CUDA; OOM.
  */
 ftcg_status_t ftcg_weights(ftcg_plan_t plan, double* d_alpha_out, ftcg_stream_t stream);

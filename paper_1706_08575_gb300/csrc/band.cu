@@ -24,8 +24,8 @@
 //
 // The FP64 pipe (2 multiply-adds per SM and clock) bounds all of it, so the design counts FP64
 // instructions. Tiny configuration (M = 4096, r = 5), us: rho 4680 as a complex matrix with two
-// sinpi and a sincospi per axis and entry, here 1017; the band of its square 1684 (one warp per
-// complex entry, every row read 18 times), here 390 (151 M multiply-adds take 240 at the pipe's
+// sinpi and a sincospi per axis and entry, here 928; the band of its square 1684 (one warp per
+// complex entry, every row read 18 times), here 398 (151 M multiply-adds take 240 at the pipe's
 // rate); solve 90, here 43.
 
 #include <cmath>

@@ -25,9 +25,9 @@
 //
 // This FP64 route serves what weights_split.cu does not take (split_lag_side there has the rule): lag
 // grids above 8192, windows whose truncation is below what two-float arithmetic resolves,
-// oversamplings and widths that could be less exact on a power-of-two grid, and rasters so uneven that
-// the pairs' rounding shows (found out by the other route, which is then lost time: 5 to 15 %). The other is faster (large
-// ping: 4.97 ms here, about 1.1 there).
+// oversamplings and widths that could be less exact on a power-of-two grid, and rasters so uneven
+// that the pairs' rounding shows (found out by the other route, which is then lost time: 5 to 35 %).
+// The other is faster (large ping: 4.97 ms here, about 1.1 there).
 
 #include <cuda_runtime.h>
 

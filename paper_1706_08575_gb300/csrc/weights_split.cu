@@ -7,8 +7,9 @@
 // integers (exactly, so the sums of a tile do not depend on their order) in shared memory, and the
 // transforms and the interpolation carry FP32 pairs (about 2^-46 relative to the largest term). The
 // window's own truncation exp(-beta) is larger than all of that, which is the condition on which
-// compute_weights takes this route: against brute-force sums both routes are off by the same
-// (2.3e-12 on the large ping, 7.2e-12 on a small one).
+// compute_weights takes this route (split_lag_side, kUneven). Rms error against pair-by-pair FP64 sums on
+// 60 polar rasters (N = 64..1024, M = 1 k..2 M, sigma = 2, w = 12): 1.00 to 1.02 times the FP64 route's at
+// N a power of two (large ping 2.3e-12), 0.01 to 0.9 times elsewhere, where this lag grid is finer.
 //
 // Steps (lag grid transposed, [x][y]: a tile's cells and a transform's line are contiguous in y):
 //   k_lag_origin   window polynomials, lag weights times window divisions (first blocks); 46-bit

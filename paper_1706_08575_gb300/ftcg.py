@@ -199,7 +199,7 @@ class Plan:
 
     # --- the operations --------------------------------------------------------------------
     def weights(self, out=None, stream=None):
-        """Exact FTCG weights (FP64, acquisition order); also installed in the plan."""
+        """Exact FTCG weights (float64, acquisition order); also installed in the plan."""
         import torch
         if out is None:
             out = torch.empty(self.M, dtype=torch.float64, device=self.device)

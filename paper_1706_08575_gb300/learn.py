@@ -1,6 +1,6 @@
 """Training and use of the weight-predicting network (argument marshalling around libftcg).
 
-Labels are the exact FTCG weights of each training geometry (ftcg_weights, FP64 on the device);
+Labels are the exact FTCG weights of each training geometry (ftcg_weights, float64);
 features come from ftcg_features; every forward, backward and Adam step runs in the library's
 BF16 tensor-core kernels. PyTorch only holds device buffers and draws batch indices.
 """
